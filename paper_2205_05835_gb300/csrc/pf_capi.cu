@@ -303,16 +303,47 @@ struct ImplT final : Impl {
         if (DIM == 3 && sizeof(T) == sizeof(float) && prm.stage_kernel == 0)
             ph.fused_stage = stage_fused_ok(g, ph) ? 1 : 0;
         for (int d = 0; d < 3; ++d) uN[d] = uS[d] = uStar[d] = accu[d] = nrm[d] = nullptr;
-        // multigrid hierarchy geometry
+        build_levels(false);
+    }
+
+    // Geometry of the multigrid hierarchy: every axis of 2 cells or more is
+    // halved (an odd one to floor(n / 2), its last coarse cell taking three
+    // children; one cell along an axis couples to nothing there), until every
+    // axis has at most 3 cells. Any size reaches a bottom level that a few
+    // sweeps solve; a hierarchy that stops at the first odd or short axis needs
+    // 4 n^2 sweeps of an n-cell axis there (a 160 x 120 x 72 step spent 135 of
+    // its 143 ms in the 20 x 15 x 9 bottom level, 200 x 136 262 of 266 ms in
+    // 25 x 17). Keeping a short axis uncoarsened instead of taking it to one
+    // cell leaves its coupling dominant and point sweeps stall (7 x 63 to 1e-9: 72
+    // iterations, against fewer than 34).
+    // even_only: halvings of even axes alone (the smaller workspace of
+    // pf_poisson_solve_static at its capacity limit).
+    void build_levels(bool even_only) {
         H.nlev = 1;
         H.lev[0].g = g;
-        while (H.nlev < kMaxLevels) {
-            const Dims& f = H.lev[H.nlev - 1].g;
-            bool ok = (f.nx % 2 == 0) && (f.ny % 2 == 0) && (DIM == 2 || f.nz % 2 == 0) &&
-                      f.nx >= 4 && f.ny >= 4 && (DIM == 2 || f.nz >= 4);
-            if (!ok) break;
-            H.lev[H.nlev].g = make_dims(f.nx / 2, f.ny / 2, DIM == 3 ? f.nz / 2 : 1, f.h * 2.0);
-            H.lev[H.nlev].g.wall_y = f.wall_y;
+        for (int d = 0; d < 3; ++d) H.lev[0].lastw[d] = 1.f;
+        for (;;) {
+            MGLevel<T>& F = H.lev[H.nlev - 1];
+            const int n[3] = {F.g.nx, F.g.ny, F.g.nz};
+            int m[3] = {n[0], n[1], n[2]};
+            bool any = false, all_even = true;
+            for (int d = 0; d < 3; ++d) {
+                F.cf[d] = 1;
+                if (d >= DIM) continue;
+                if (n[d] < 4 || n[d] % 2 != 0) all_even = false;
+                if (n[d] >= 4) any = true;
+                if (n[d] >= 2) {
+                    F.cf[d] = 2;
+                    m[d] = n[d] / 2;
+                }
+            }
+            if (H.nlev == kMaxLevels || !any || (even_only && !all_even)) break;
+            MGLevel<T>& C = H.lev[H.nlev];
+            C.g = make_dims(m[0], m[1], m[2], F.g.h * 2.0);
+            C.g.wall_y = F.g.wall_y;
+            for (int d = 0; d < 3; ++d)
+                C.lastw[d] = F.cf[d] == 1 ? F.lastw[d]
+                                          : 0.5f * (F.lastw[d] + (n[d] % 2 ? 2.f : 1.f));
             ++H.nlev;
         }
         for (int l = 0; l < kMaxLevels; ++l) H.lev[l].x2 = nullptr;
@@ -325,8 +356,10 @@ struct ImplT final : Impl {
         const Dims& cg = H.lev[H.nlev - 1].g;
         int nmax = cg.nx > cg.ny ? cg.nx : cg.ny;
         if (cg.nz > nmax) nmax = cg.nz;
-        int sweeps = 4 * nmax * nmax;
-        H.coarse_sweeps = sweeps < 8 ? 8 : (sweeps > 2000 ? 2000 : sweeps);
+        // two or three cells an axis: Gauss-Seidel reduces the slowest mode by
+        // 1/4 (three cells in 3D, uniform density) or more a sweep
+        const int sweeps = nmax <= 2 ? 4 : (nmax == 3 ? 5 : 4 * nmax * nmax);
+        H.coarse_sweeps = sweeps > 2000 ? 2000 : sweeps;
     }
 
     bool owns_host = false;
@@ -433,7 +466,8 @@ struct ImplT final : Impl {
         // on a pointer: the sizing pass carves from a null base.)
         if (DIM == 3 && sizeof(T) == sizeof(float))
             for (int l = 1; l < H.first_coarse && l <= kDensityLevels; ++l)
-                H.rhoc[l] = sweep3d_ok(H.lev[l].g) ? cv.take<float>(H.lev[l].g.ncell) : nullptr;
+                H.rhoc[l] = sweep3d_ok(H.lev[l].g) && sweep3d_ok(H.lev[l - 1].g)
+                                ? cv.take<float>(H.lev[l].g.ncell) : nullptr;
         rb.part = cv.take<double>(kRedPart);
         rb.counter = cv.take<unsigned int>(4);
         sc = cv.take<CGScalars>(1);
@@ -1489,6 +1523,13 @@ pf_status run_static_solve(const pf_params& prm, cudaStream_t st, void* scratch,
     if (!err.empty()) return PF_ERR_INVALID;
     Carver size_cv{nullptr};
     im.carve_solver_only(size_cv);
+    if (size_cv.off > (size_t)PF_STATIC_SCRATCH_BYTES) {
+        // odd sizes coarsened add levels: a grid that fits without them is solved
+        // without them
+        im.build_levels(true);
+        size_cv.off = 0;
+        im.carve_solver_only(size_cv);
+    }
     if (size_cv.off > (size_t)PF_STATIC_SCRATCH_BYTES) {
         err = "grid too large for the static scratch of pf_poisson_solve_static (" +
               std::to_string(size_cv.off) + " bytes needed, " +

@@ -224,6 +224,19 @@ __device__ __forceinline__ void for_cells(const Dims& g, F f) {
     }
 }
 
+// Classes of a Gauss-Seidel sweep on a periodic level: colour (i + j + k) % 2
+// plus 2 s, s the number of axes of odd size along which the cell is the last
+// one. Two neighbours never share a class: across an odd axis's seam, where
+// their colours agree, s differs by one. Even levels have the two colours only.
+__host__ __device__ __forceinline__ int odd_axis(int n) { return n > 1 ? (n & 1) : 0; }
+__host__ __device__ __forceinline__ int gs_classes(const Dims& g) {
+    return 2 + 2 * (odd_axis(g.nx) + odd_axis(g.ny) + odd_axis(g.nz));
+}
+__device__ __forceinline__ int gs_seams(const Dims& g, int i, int j, int k) {
+    return (odd_axis(g.nx) && i == g.nx - 1) + (odd_axis(g.ny) && j == g.ny - 1) +
+           (odd_axis(g.nz) && k == g.nz - 1);
+}
+
 // Same, over the cells of one colour ((i + j + k) % 2 == color).
 template <typename F>
 __device__ __forceinline__ void for_color_cells(const Dims& g, int color, F f) {

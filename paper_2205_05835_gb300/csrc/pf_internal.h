@@ -114,7 +114,11 @@ struct CGScalars {
     int it_in;        // iterations of the current inner solve (device-driven loops)
 };
 
-// One multigrid level of the preconditioner.
+// One multigrid level of the preconditioner. Its equations are the finite-volume
+// ones over the level's cells, divided by the nominal cell volume: the sum over
+// the faces of beta ih2 (x_c - x_q) = f, with beta a coefficient that carries
+// the face's area and the distance of the two centres (exactly 1/rho_f's mean
+// on uniform levels).
 template <typename T>
 struct MGLevel {
     Dims g;
@@ -122,6 +126,12 @@ struct MGLevel {
     T* f;          // right-hand side
     T* beta[3];    // face coefficients 1/rho_f (nullptr on level 0: computed from phi)
     T* x2;         // second correction buffer for out-of-place sweeps (nullptr: in place)
+    // Coarsening to the next level: factor cf[d] (2, or 1 where an axis has one
+    // cell) and n[d] / cf[d] coarse cells, the last of which takes three
+    // children where n[d] is odd. lastw[d]: width of the last cell
+    // along d over the level's nominal width (1 up to the first odd size).
+    int cf[3];
+    float lastw[3];
 };
 
 

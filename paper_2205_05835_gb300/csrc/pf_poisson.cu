@@ -81,42 +81,119 @@ __device__ __forceinline__ void gs_cell(const MGLevel<T>& L, const T* __restrict
     L.x[idx] = divq(L.f[idx] + off, diag);
 }
 
-// f_{l+1}(I) = mean of the residual of the 2^d children of coarse cell I
-template <typename T, int DIM>
+// Children of coarse cell I along axis d of level F: cells [c cf, c cf + count).
+template <typename T>
+__device__ __forceinline__ int child_count(const MGLevel<T>& F, int d, int nf, int nc, int I) {
+    return F.cf[d] == 1 ? 1 : (I == nc - 1 ? nf - 2 * I : 2);
+}
+
+// f_{l+1}(I) = sum of the residuals of the children of coarse cell I over the
+// nominal number of children (their mean on even levels)
+// (UNI: every coarse cell has two children along each axis)
+template <typename T, int DIM, bool UNI>
 __device__ __forceinline__ void restrict_cell(const MGLevel<T>& F, const MGLevel<T>& C,
                                               const T* __restrict__ phi, const Phys& ph, int ci,
                                               int cj, int ck, int I) {
     T s = T(0);
+    if constexpr (UNI) {
 #pragma unroll
-    for (int a = 0; a < (DIM == 3 ? 2 : 1); ++a)
+        for (int a = 0; a < (DIM == 3 ? 2 : 1); ++a)
 #pragma unroll
-        for (int b = 0; b < 2; ++b)
+            for (int b = 0; b < 2; ++b)
 #pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const int fi = 2 * ci + e, fj = 2 * cj + b, fk = DIM == 3 ? 2 * ck + a : 0;
-                s += residual_at<T, DIM>(F, phi, ph, fi, fj, fk, (fk * F.g.ny + fj) * F.g.nx + fi);
-            }
-    C.f[I] = s * T(DIM == 3 ? 0.125 : 0.25);
+                for (int e = 0; e < 2; ++e) {
+                    const int fi = 2 * ci + e, fj = 2 * cj + b, fk = DIM == 3 ? 2 * ck + a : 0;
+                    s += residual_at<T, DIM>(F, phi, ph, fi, fj, fk,
+                                             (fk * F.g.ny + fj) * F.g.nx + fi);
+                }
+        C.f[I] = s * T(DIM == 3 ? 0.125 : 0.25);
+    } else {
+        const int ex = child_count(F, 0, F.g.nx, C.g.nx, ci);
+        const int ey = child_count(F, 1, F.g.ny, C.g.ny, cj);
+        const int ez = DIM == 3 ? child_count(F, 2, F.g.nz, C.g.nz, ck) : 1;
+        for (int a = 0; a < ez; ++a)
+            for (int b = 0; b < ey; ++b)
+                for (int e = 0; e < ex; ++e) {
+                    const int fi = F.cf[0] * ci + e, fj = F.cf[1] * cj + b,
+                              fk = DIM == 3 ? F.cf[2] * ck + a : 0;
+                    s += residual_at<T, DIM>(F, phi, ph, fi, fj, fk,
+                                             (fk * F.g.ny + fj) * F.g.nx + fi);
+                }
+        const int vol = F.cf[0] * F.cf[1] * (DIM == 3 ? F.cf[2] : 1);
+        C.f[I] = s * (T(1) / T(vol));
+    }
+}
+
+// Linear interpolation along one axis: fine cell i lies in coarse cell I0 and
+// takes weight w of the coarse neighbour I1 on its side, 1 - w of I0: 1/4 and
+// 3/4 between cells of nominal width, from the centres' distances beside a
+// last cell of another width, 1 - w = 1 on an axis that is not coarsened.
+template <typename T>
+__device__ __forceinline__ void interp_axis(int i, int nf, int nc, int cf, float qf, float qc,
+                                            int& I0, int& I1, T& w) {
+    if (cf == 1) {
+        I0 = I1 = i;
+        w = T(0);
+        return;
+    }
+    I0 = i >> 1;
+    if (qc == 1.f) {
+        I1 = wrapi(I0 + ((i & 1) ? 1 : -1), nc);
+        w = T(0.25);
+        return;
+    }
+    if (I0 > nc - 1) I0 = nc - 1;
+    const float wp = 2.f * (I0 == nc - 1 ? qc : 1.f);
+    const float o = float(i - 2 * I0) + 0.5f * (i == nf - 1 ? qf : 1.f) - 0.5f * wp;
+    I1 = wrapi(I0 + (o >= 0.f ? 1 : -1), nc);
+    w = T(fabsf(o) / (0.5f * wp + (I1 == nc - 1 ? qc : 1.f)));
 }
 
 // x_l(i) += linear interpolation of x_{l+1} (weights 3/4, 1/4 per axis)
-template <typename T, int DIM>
+// (UNI: both levels uniform, every axis halved)
+template <typename T, int DIM, bool UNI>
 __device__ __forceinline__ void prolong_cell(const MGLevel<T>& F, const MGLevel<T>& C, int i, int j,
                                              int k, int idx) {
-    const int I0 = i >> 1, J0 = j >> 1, K0 = DIM == 3 ? k >> 1 : 0;
-    const int I1 = wrapi(I0 + ((i & 1) ? 1 : -1), C.g.nx);
-    const int J1 = wrapi(J0 + ((j & 1) ? 1 : -1), C.g.ny);
-    const int K1 = DIM == 3 ? wrapi(K0 + ((k & 1) ? 1 : -1), C.g.nz) : 0;
     const T* xc = C.x;
     auto at = [&](int a, int b, int c) { return xc[(c * C.g.ny + b) * C.g.nx + a]; };
-    T v = T(0.5625) * at(I0, J0, K0) + T(0.1875) * (at(I1, J0, K0) + at(I0, J1, K0)) +
-          T(0.0625) * at(I1, J1, K0);
-    if (DIM == 3) {
-        T v1 = T(0.5625) * at(I0, J0, K1) + T(0.1875) * (at(I1, J0, K1) + at(I0, J1, K1)) +
-               T(0.0625) * at(I1, J1, K1);
-        v = T(0.75) * v + T(0.25) * v1;
+    if constexpr (UNI) {
+        const int I0 = i >> 1, J0 = j >> 1, K0 = DIM == 3 ? k >> 1 : 0;
+        const int I1 = wrapi(I0 + ((i & 1) ? 1 : -1), C.g.nx);
+        const int J1 = wrapi(J0 + ((j & 1) ? 1 : -1), C.g.ny);
+        T v = T(0.5625) * at(I0, J0, K0) + T(0.1875) * (at(I1, J0, K0) + at(I0, J1, K0)) +
+              T(0.0625) * at(I1, J1, K0);
+        if (DIM == 3) {
+            const int K1 = wrapi(K0 + ((k & 1) ? 1 : -1), C.g.nz);
+            const T v1 = T(0.5625) * at(I0, J0, K1) +
+                         T(0.1875) * (at(I1, J0, K1) + at(I0, J1, K1)) +
+                         T(0.0625) * at(I1, J1, K1);
+            v = T(0.75) * v + T(0.25) * v1;
+        }
+        F.x[idx] += v;
+    } else {
+        int I0, I1, J0, J1, K0 = 0, K1 = 0;
+        T wi, wj, wk = T(0);
+        interp_axis<T>(i, F.g.nx, C.g.nx, F.cf[0], F.lastw[0], C.lastw[0], I0, I1, wi);
+        interp_axis<T>(j, F.g.ny, C.g.ny, F.cf[1], F.lastw[1], C.lastw[1], J0, J1, wj);
+        if (DIM == 3)
+            interp_axis<T>(k, F.g.nz, C.g.nz, F.cf[2], F.lastw[2], C.lastw[2], K0, K1, wk);
+        const T w00 = (T(1) - wi) * (T(1) - wj), w10 = wi * (T(1) - wj), w01 = (T(1) - wi) * wj,
+                w11 = wi * wj;
+        T v = w00 * at(I0, J0, K0) + w10 * at(I1, J0, K0) + w01 * at(I0, J1, K0) + w11 * at(I1, J1, K0);
+        if (DIM == 3) {
+            const T v1 = w00 * at(I0, J0, K1) + w10 * at(I1, J0, K1) + w01 * at(I0, J1, K1) +
+                         w11 * at(I1, J1, K1);
+            v = (T(1) - wk) * v + wk * v1;
+        }
+        F.x[idx] += v;
     }
-    F.x[idx] += v;
+}
+
+template <typename T, int DIM>
+__host__ __device__ __forceinline__ bool uniform_pair(const MGLevel<T>& F, const MGLevel<T>& C) {
+    bool u = true;
+    for (int d = 0; d < DIM; ++d) u = u && F.cf[d] == 2 && C.lastw[d] == 1.f;
+    return u;
 }
 
 __device__ __forceinline__ bool inner_stopped(const CGScalars* sc) { return sc->done || sc->idone; }
@@ -126,36 +203,42 @@ __device__ __forceinline__ bool inner_stopped(const CGScalars* sc) { return sc->
 // ---------------------------------------------------------------------------
 template <typename T, int DIM>
 __global__ void __launch_bounds__(kThreads)
-k_gs(MGLevel<T> L, const T* __restrict__ phi, Phys ph, int color, int zero_start,
+k_gs(MGLevel<T> L, const T* __restrict__ phi, Phys ph, int cls, int zero_start,
      const CGScalars* sc) {
     if (inner_stopped(sc)) return;
+    const int color = cls & 1, seams = cls >> 1;
+    const bool odd = gs_classes(L.g) > 2;
     if (zero_start) {
-        // both colours: active colour x = f/diag, the other 0
+        // every class: the active one x = f/diag, the others 0
         for_cells(L.g, [&](int i, int j, int k, int idx) {
-            if (((i + j + k) & 1) == color) gs_cell<T, DIM>(L, phi, ph, i, j, k, idx, true);
+            if (((i + j + k) & 1) == color && (!odd || gs_seams(L.g, i, j, k) == seams))
+                gs_cell<T, DIM>(L, phi, ph, i, j, k, idx, true);
             else L.x[idx] = T(0);
         });
     } else {
         for_color_cells(L.g, color, [&](int i, int j, int k, int idx) {
-            gs_cell<T, DIM>(L, phi, ph, i, j, k, idx, false);
+            if (!odd || gs_seams(L.g, i, j, k) == seams)
+                gs_cell<T, DIM>(L, phi, ph, i, j, k, idx, false);
         });
     }
 }
 
-template <typename T, int DIM>
+template <typename T, int DIM, bool UNI>
 __global__ void __launch_bounds__(kThreads)
 k_restrict(MGLevel<T> F, MGLevel<T> C, const T* __restrict__ phi, Phys ph, const CGScalars* sc) {
     if (inner_stopped(sc)) return;
     for_cells(C.g, [&](int i, int j, int k, int I) {
-        restrict_cell<T, DIM>(F, C, phi, ph, i, j, k, I);
+        restrict_cell<T, DIM, UNI>(F, C, phi, ph, i, j, k, I);
     });
 }
 
-template <typename T, int DIM>
+template <typename T, int DIM, bool UNI>
 __global__ void __launch_bounds__(kThreads)
 k_prolong(MGLevel<T> F, MGLevel<T> C, const CGScalars* sc) {
     if (inner_stopped(sc)) return;
-    for_cells(F.g, [&](int i, int j, int k, int idx) { prolong_cell<T, DIM>(F, C, i, j, k, idx); });
+    for_cells(F.g, [&](int i, int j, int k, int idx) {
+        prolong_cell<T, DIM, UNI>(F, C, i, j, k, idx);
+    });
 }
 
 // 3D, even nx: one thread per pair of fine cells (2I, 2I+1) of a row, which
@@ -272,24 +355,31 @@ k_prolong_zm(MGLevel<float> F, MGLevel<float> C, int kc, const CGScalars* sc) {
     }
 }
 
-// coarse face coefficients: mean of the 2^(d-1) fine faces on each coarse face
+// Coarse face coefficients: the sum of the fine faces that a coarse face
+// covers, scaled by the nominal volume ratio and by the ratio of the centres'
+// distances (the mean of the 2^(d-1) fine faces where both levels are uniform).
 template <typename T, int DIM>
 __global__ void __launch_bounds__(kThreads)
 k_coarsen_beta(MGLevel<T> F, MGLevel<T> C, const T* __restrict__ phi, Phys ph) {
+    const int fn[3] = {F.g.nx, F.g.ny, F.g.nz}, cn[3] = {C.g.nx, C.g.ny, C.g.nz};
+    const int vol = F.cf[0] * F.cf[1] * (DIM == 3 ? F.cf[2] : 1);
     for_cells(C.g, [&](int ci, int cj, int ck, int I) {
+        const int cc[3] = {ci, cj, ck};
+        int cnt[3] = {1, 1, 1};
+#pragma unroll
+        for (int d = 0; d < DIM; ++d) cnt[d] = child_count(F, d, fn[d], cn[d], cc[d]);
 #pragma unroll
         for (int d = 0; d < DIM; ++d) {
+            const int e1 = (d + 1) % DIM, e2 = (d + 2) % 3;
+            const int n1 = cnt[e1], n2 = DIM == 3 ? cnt[e2] : 1;
             T s = T(0);
-#pragma unroll
-            for (int a = 0; a < 2; ++a)
-#pragma unroll
-                for (int b = 0; b < (DIM == 3 ? 2 : 1); ++b) {
+            for (int a = 0; a < n1; ++a)
+                for (int b = 0; b < n2; ++b) {
                     int o[3] = {0, 0, 0};
-                    const int e1 = (d + 1) % DIM, e2 = (d + 2) % 3;
                     o[e1] = a;
                     if (DIM == 3) o[e2] = b;
-                    const int fi = 2 * ci + o[0], fj = 2 * cj + o[1],
-                              fk = DIM == 3 ? 2 * ck + o[2] : 0;
+                    const int fi = F.cf[0] * ci + o[0], fj = F.cf[1] * cj + o[1],
+                              fk = DIM == 3 ? F.cf[2] * ck + o[2] : 0;
                     const int fidx = (fk * F.g.ny + fj) * F.g.nx + fi;
                     T bf;
                     if (F.beta[0] == nullptr) {
@@ -303,7 +393,16 @@ k_coarsen_beta(MGLevel<T> F, MGLevel<T> C, const T* __restrict__ phi, Phys ph) {
                     }
                     s += bf;
                 }
-            C.beta[d][I] = s * T(DIM == 3 ? 0.25 : 0.5);
+            // distances of the two centres across the face, in fine nominal
+            // widths: cell 0's lower neighbour is the last cell
+            const int c0 = cc[d], f0 = F.cf[d] * c0;
+            const float qf = F.lastw[d], qc = C.lastw[d];
+            const float df = 0.5f * ((f0 == fn[d] - 1 ? qf : 1.f) +
+                                     ((f0 == 0 ? fn[d] - 1 : f0 - 1) == fn[d] - 1 ? qf : 1.f));
+            const float dc = 0.5f * float(F.cf[d]) *
+                             ((c0 == cn[d] - 1 ? qc : 1.f) +
+                              ((c0 == 0 ? cn[d] - 1 : c0 - 1) == cn[d] - 1 ? qc : 1.f));
+            C.beta[d][I] = cn[d] == 1 ? T(0) : s * T(4.f * df / (dc * float(vol)));
         }
     });
 }
@@ -391,16 +490,18 @@ template void launch_beta0_32<3>(const Dims&, const Phys&, const float*, float* 
 constexpr int kCoarseThreads = 1024;
 constexpr size_t kCoarseSmemMax = 200 * 1024;   // staged coarse hierarchy, bytes
 
-// One colour of a red-black sweep over a (small) level by threads t0, t0 + nt,
+// One class of a Gauss-Seidel sweep over a (small) level by threads t0, t0 + nt,
 // ...: item q = (row, m) with cell i = 2 m + parity(row) of the colour; all:
-// the other colour's cell of the pair is zeroed. Rows and positions come from
+// the cells of the other classes are zeroed. Rows and positions come from
 // float reciprocals: (q + 1/2) / n lies at least 1/(2n) from an integer and
 // the two roundings move it by at most (q + 1/2) 2^-23 / n, so the quotient
 // truncates exactly for q < 2^22 (levels up to 2^20 cells run here).
 template <typename T, int DIM>
-__device__ __forceinline__ void cta_cells(const Dims& g, int color, bool all, const MGLevel<T>& L,
+__device__ __forceinline__ void cta_cells(const Dims& g, int cls, bool all, const MGLevel<T>& L,
                                           const T* phi, const Phys& ph, bool zero_start,
                                           int t0, int nt) {
+    const int color = cls & 1, seams = cls >> 1;
+    const bool odd = gs_classes(g) > 2;
     const int nhx = (g.nx + 1) >> 1;
     const int rows = g.ny * g.nz;
     const int items = rows * nhx;
@@ -413,7 +514,11 @@ __device__ __forceinline__ void cta_cells(const Dims& g, int color, bool all, co
         const int par = (j + k + color) & 1;
         const int i = 2 * m + par;
         const int base = r * g.nx;
-        if (i < g.nx) gs_cell<T, DIM>(L, phi, ph, i, j, k, base + i, zero_start);
+        if (i < g.nx) {
+            if (!odd || gs_seams(g, i, j, k) == seams)
+                gs_cell<T, DIM>(L, phi, ph, i, j, k, base + i, zero_start);
+            else if (all) L.x[base + i] = T(0);
+        }
         if (all) {
             const int io = 2 * m + (1 - par);
             if (io < g.nx) L.x[base + io] = T(0);
@@ -444,17 +549,19 @@ __device__ __forceinline__ void coarse_vcycle_body(MGLevel<T>* L_, int l0, int l
     // down
     for (int l = l0; l < lb; ++l) {
         const MGLevel<T>& L = L_[l];
-        for (int s = 0; s < pre; ++s) {
-            cta_cells<T, DIM>(L.g, 0, s == 0, L, phi, ph, s == 0, tid, nt);
-            __syncthreads();
-            cta_cells<T, DIM>(L.g, 1, false, L, phi, ph, false, tid, nt);
-            __syncthreads();
-        }
+        const int ncl = gs_classes(L.g);
+        for (int s = 0; s < pre; ++s)
+            for (int c = 0; c < ncl; ++c) {
+                cta_cells<T, DIM>(L.g, c, s == 0 && c == 0, L, phi, ph, s == 0 && c == 0, tid, nt);
+                __syncthreads();
+            }
         const MGLevel<T>& C = L_[l + 1];
         const float cix = 1.0f / float(C.g.nx), ciy = 1.0f / float(C.g.ny);
+        const bool uni = uniform_pair<T, DIM>(L, C);
         for (int I = tid; I < C.g.ncell; I += nt) {
             Cell c = decode_small(I, C.g, cix, ciy);
-            restrict_cell<T, DIM>(L, C, phi, ph, c.i, c.j, c.k, I);
+            if (uni) restrict_cell<T, DIM, true>(L, C, phi, ph, c.i, c.j, c.k, I);
+            else restrict_cell<T, DIM, false>(L, C, phi, ph, c.i, c.j, c.k, I);
         }
         __syncthreads();
     }
@@ -475,28 +582,31 @@ __device__ __forceinline__ void coarse_vcycle_body(MGLevel<T>* L_, int l0, int l
         const T mean = T(red[0]);
         for (int i = tid; i < L.g.ncell; i += nt) L.f[i] -= mean;
         __syncthreads();
-        for (int s2 = 0; s2 < coarse_sweeps; ++s2) {
-            cta_cells<T, DIM>(L.g, 0, s2 == 0, L, phi, ph, s2 == 0, tid, nt);
-            __syncthreads();
-            cta_cells<T, DIM>(L.g, 1, false, L, phi, ph, false, tid, nt);
-            __syncthreads();
-        }
+        const int ncl = gs_classes(L.g);
+        for (int s2 = 0; s2 < coarse_sweeps; ++s2)
+            for (int c = 0; c < ncl; ++c) {
+                cta_cells<T, DIM>(L.g, c, s2 == 0 && c == 0, L, phi, ph, s2 == 0 && c == 0, tid,
+                                  nt);
+                __syncthreads();
+            }
     }
     // up
     for (int l = lb - 1; l >= l0; --l) {
         const MGLevel<T>& L = L_[l];
         const float fix = 1.0f / float(L.g.nx), fiy = 1.0f / float(L.g.ny);
+        const bool uni = uniform_pair<T, DIM>(L, L_[l + 1]);
         for (int i = tid; i < L.g.ncell; i += nt) {
             Cell c = decode_small(i, L.g, fix, fiy);
-            prolong_cell<T, DIM>(L, L_[l + 1], c.i, c.j, c.k, i);
+            if (uni) prolong_cell<T, DIM, true>(L, L_[l + 1], c.i, c.j, c.k, i);
+            else prolong_cell<T, DIM, false>(L, L_[l + 1], c.i, c.j, c.k, i);
         }
         __syncthreads();
-        for (int s = 0; s < post; ++s) {
-            cta_cells<T, DIM>(L.g, 1, false, L, phi, ph, false, tid, nt);
-            __syncthreads();
-            cta_cells<T, DIM>(L.g, 0, false, L, phi, ph, false, tid, nt);
-            __syncthreads();
-        }
+        const int ncl = gs_classes(L.g);
+        for (int s = 0; s < post; ++s)
+            for (int c = ncl - 1; c >= 0; --c) {
+                cta_cells<T, DIM>(L.g, c, false, L, phi, ph, false, tid, nt);
+                __syncthreads();
+            }
     }
 }
 
@@ -628,10 +738,10 @@ T* launch_vcycle(const Phys& ph, const T* phi, MGHier<T>& H, const CGScalars* sc
     auto rho_ready_of = [&](int l) { return l == 0 ? rho_ready : 1; };
     T* fin[kMaxLevels];   // buffer holding each level's result
     for (int l = l0; l < H.nlev; ++l) fin[l] = H.lev[l].x;
-    auto gs = [&](const MGLevel<T>& L, int lvl, int color, int zero) {
+    auto gs = [&](const MGLevel<T>& L, int lvl, int cls, int zero) {
         pr->begin(lvl == 0 ? KC_GS0 : KC_GS);
-        k_gs<T, DIM><<<row_grid(L.g, kThreads, 1 << 30), kThreads, 0, s>>>(L, phi, ph, color,
-                                                                          zero, sc);
+        k_gs<T, DIM><<<row_grid(L.g, kThreads, 1 << 30), kThreads, 0, s>>>(L, phi, ph, cls, zero,
+                                                                          sc);
         pr->end();
     };
     T* pre_buf[kMaxLevels];
@@ -658,10 +768,8 @@ T* launch_vcycle(const Phys& ph, const T* phi, MGHier<T>& H, const CGScalars* sc
                 pre_buf[l] = cur;
             }
         } else {
-            for (int p = 0; p < H.pre; ++p) {
-                gs(L, l, 0, p == 0);
-                gs(L, l, 1, 0);
-            }
+            for (int p = 0; p < H.pre; ++p)
+                for (int c = 0; c < gs_classes(L.g); ++c) gs(L, l, c, p == 0 && c == 0);
             pre_buf[l] = L.x;
         }
         L.x = pre_buf[l];
@@ -675,9 +783,13 @@ T* launch_vcycle(const Phys& ph, const T* phi, MGHier<T>& H, const CGScalars* sc
                 done_r = true;
             }
         }
-        if (!done_r)
-            k_restrict<T, DIM><<<row_grid(H.lev[l + 1].g, kThreads, 1 << 30), kThreads, 0, s>>>(
-                L, H.lev[l + 1], phi, ph, sc);
+        if (!done_r) {
+            const int gr = row_grid(H.lev[l + 1].g, kThreads, 1 << 30);
+            if (uniform_pair<T, DIM>(L, H.lev[l + 1]))
+                k_restrict<T, DIM, true><<<gr, kThreads, 0, s>>>(L, H.lev[l + 1], phi, ph, sc);
+            else
+                k_restrict<T, DIM, false><<<gr, kThreads, 0, s>>>(L, H.lev[l + 1], phi, ph, sc);
+        }
         pr->end();
     }
     pr->begin(KC_COARSE);
@@ -741,12 +853,14 @@ T* launch_vcycle(const Phys& ph, const T* phi, MGHier<T>& H, const CGScalars* sc
         } else {
             L.x = pre_buf[l];
             pr->begin(KC_PROLONG);
-            k_prolong<T, DIM><<<row_grid(L.g, kThreads, 1 << 30), kThreads, 0, s>>>(L, C, sc);
+            const int gr = row_grid(L.g, kThreads, 1 << 30);
+            if (uniform_pair<T, DIM>(L, C))
+                k_prolong<T, DIM, true><<<gr, kThreads, 0, s>>>(L, C, sc);
+            else
+                k_prolong<T, DIM, false><<<gr, kThreads, 0, s>>>(L, C, sc);
             pr->end();
-            for (int p = 0; p < H.post; ++p) {
-                gs(L, l, 1, 0);
-                gs(L, l, 0, 0);
-            }
+            for (int p = 0; p < H.post; ++p)
+                for (int c = gs_classes(L.g) - 1; c >= 0; --c) gs(L, l, c, 0);
             fin[l] = L.x;
         }
     }

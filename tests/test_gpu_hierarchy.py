@@ -1,0 +1,65 @@
+"""Pressure solves on grids whose multigrid hierarchy has odd sizes, short axes
+or unequal axes, against the oracle's exact solve of the same operator."""
+import numpy as np
+import pytest
+
+import pf_inputs as I
+from oracle import pf_oracle as O
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pf():
+    import torch
+
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__ as g
+
+    g.build()
+    import paper_2205_05835_gb300 as pf
+
+    return pf
+
+
+def beta32(phi, g, p):
+    """The mixed path's float32 face coefficients, operation by operation."""
+    f = np.float32
+    c = np.clip(phi.astype(f), f(0), f(1))
+    rho = f(p["rho_out"]) + (f(p["rho_in"]) - f(p["rho_out"])) * c
+    return [(f(1) / (f(0.5) * (rho + np.roll(rho, 1, g.axis(d))))).astype(np.float64)
+            for d in range(g.dim)]
+
+
+SIZES = [(4, 4), (5, 4), (7, 63), (33, 31), (61, 45), (64, 64), (100, 36), (200, 6), (130, 66),
+         (6, 5, 4), (9, 7, 5), (20, 15, 9), (24, 4, 50), (17, 18, 13), (32, 20, 12)]
+
+
+@pytest.mark.parametrize("n", SIZES)
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_solve_on_any_size(pf, n, precision):
+    rtol = 1e-11 if precision == "fp64" else 1e-9
+    p = I.small_case(dim=len(n), n=n[0], precision=precision, poisson_rtol=rtol, R=0.2)
+    p["n"] = tuple(n) + (1,) * (3 - len(n))
+    p = I.finalize(p)
+    po = O.params_from(p)
+    g = O.Grid(len(n), n, p["L"])
+    phi = np.clip(O.initial_phi(po) + 0.1 * (I.noise(g.shape, 5) - 0.5), 0.0, 1.0)
+    phi = phi.astype(np.float32).astype(np.float64)
+    rhs = I.noise(g.shape, 6) - 0.5
+    sim = pf.Simulation(p, phi0=phi)
+    x, iters, rel, status = sim.poisson_solve(rhs)
+    sim.close()
+    beta = O.face_beta(phi, g, po) if precision == "fp64" else beta32(phi, g, p)
+    want = O.solve_poisson(beta, rhs, g)
+    assert status == 0 and rel <= rtol
+    # |x - x*| <= |r| / lambda_min <= rtol |f| / lambda_min in the 2-norm (plus the
+    # rounding of the double-float right-hand side, 2^-47, in the mixed form);
+    # lambda_min >= min beta (smallest non-zero eigenvalue of the Laplacian)
+    h = g.h
+    lam = min(b.min() for b in beta) * (2 - 2 * np.cos(2 * np.pi / max(n))) / h ** 2
+    f = rhs - rhs.mean()
+    assert np.linalg.norm(x - want) <= (1.01 * rtol + 2.0 ** -40) * np.linalg.norm(f) / lam
+    # a V-cycle that halves the error per iteration or better
+    assert iters <= np.log2(1.0 / rtol) + 4
