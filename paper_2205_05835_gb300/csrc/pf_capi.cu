@@ -10,6 +10,7 @@
 
 #include "../../include/pf.h"
 #include "pf_internal.h"
+#include "pf_solve2d.cuh"
 
 using namespace pf;
 
@@ -60,7 +61,8 @@ struct GraphBuilder {
 const char* kClassNames[KC_COUNT] = {
     "cell_pass", "stage", "gamma", "divergence", "correct", "mg_coarsen_beta", "mg_gs_level0",
     "mg_gs_coarse_levels", "mg_restrict", "mg_prolong", "mg_coarse_vcycle", "ir_residual_f64",
-    "cg_dots", "cg_dir_spmv", "cg_update", "diagnostics", "misc", "ir_addcorr", "beta0_f64"};
+    "cg_dots", "cg_dir_spmv", "cg_update", "diagnostics", "misc", "ir_addcorr", "beta0_f64",
+    "solve2d_cluster"};
 
 const double kRK4C[4] = {0.0, 0.5, 0.5, 1.0};
 const double kRK4W[4] = {1.0 / 6.0, 1.0 / 3.0, 1.0 / 3.0, 1.0 / 6.0};
@@ -364,6 +366,9 @@ struct ImplT final : Impl {
 
     bool owns_host = false;
     cudaEvent_t sleep_ev = nullptr;   // blocking-sync event (batched execution)
+
+    S2Plan s2;                 // one-launch solve of 2D grids that fit (s2_state 1; 0 not decided,
+    int s2_state = 0;          // 2 the multi-kernel solve)
 
     SweepTMA* tma = nullptr;   // tensor maps of the TMA-staged finest sweep (host object)
     SweepTMA* tmac[kMaxLevels] = {};   // the same for the coarser tiled levels
@@ -712,6 +717,18 @@ struct ImplT final : Impl {
         prof.end();
     }
 
+    T* beta_out(int d) {
+        return sizeof(T) == sizeof(double) ? reinterpret_cast<T*>(beta64[d])
+                                           : reinterpret_cast<T*>(beta32[d]);
+    }
+    bool use_solve2d() {
+        if constexpr (DIM == 2) {
+            if (s2_state == 0) s2_state = solve2d_plan<T>(H, beta_out(0) != nullptr, s2) ? 1 : 2;
+            return s2_state == 1;
+        }
+        return false;
+    }
+
     // operator setup and the first outer residual of a solve
     void solve_prologue(SolveIO<T, DIM>& io, const T* phi) {
         if (sizeof(T) == sizeof(double)) {
@@ -743,6 +760,19 @@ struct ImplT final : Impl {
     // A x = sign (b - mean b): float64 iterative refinement around inner
     // MG-preconditioned CG in T, warm start from x = p
     pf_status solve(const T* phi, double sign) {
+        if constexpr (DIM == 2) {
+            if (use_solve2d()) {
+                SolveIO<T, DIM> io = solve_io(phi, sign);
+                prof.begin(KC_SOLVE2D);
+                CK(launch_solve2d<T>(s2, g, ph, io, H, beta_out(0), beta_out(1), sc, st));
+                prof.end();
+                if (gb) return PF_OK;
+                pf_status ps = poll();
+                if (ps != PF_OK) return ps;
+                CK(cudaGetLastError());
+                return solve_status();
+            }
+        }
         if (gb) return solve_captured(phi, sign);
         SolveIO<T, DIM> io = solve_io(phi, sign);
         solve_prologue(io, phi);
@@ -855,6 +885,7 @@ struct ImplT final : Impl {
         sweep_tma_prepare();
         stage_fused_prepare();
         coarse_prepare();
+        if (DIM == 2) use_solve2d();
         // the legacy default stream cannot be captured: record on a private
         // stream (recording runs nothing); the graph replays on the context's
         cudaStream_t own = st, rec = nullptr;

@@ -440,6 +440,14 @@ __device__ __forceinline__ void df_face_term(float beta, float ch, float cl, flo
     c = __fadd_rn(c, __fadd_rn(sm.lo, __fmaf_rn(beta, t, pr.lo)));
 }
 
+// x += e (mixed path: x a double-float, hi plane and lo plane)
+__device__ __forceinline__ void df_acc(float& h, float& l, float e) {
+    const f2 s = two_sum(h, e);
+    const f2 r = two_sum(s.hi, __fadd_rn(s.lo, l));
+    h = r.hi;
+    l = r.lo;
+}
+
 inline int red_grid(int n) {
     int b = (n + kThreads - 1) / kThreads;
     return b < kRedBlocks ? (b < 1 ? 1 : b) : kRedBlocks;

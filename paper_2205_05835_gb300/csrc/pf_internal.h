@@ -252,7 +252,7 @@ struct DiagOut {
 enum KernelClass {
     KC_CELL = 0, KC_STAGE, KC_GAMMA, KC_DIV, KC_CORRECT, KC_COARSEN, KC_GS0, KC_GS,
     KC_RESTRICT, KC_PROLONG, KC_COARSE, KC_IR_RESIDUAL, KC_CG_DOTS, KC_CG_DIR, KC_CG_UPDATE,
-    KC_DIAG, KC_MISC, KC_IR_ADDCORR, KC_BETA0, KC_COUNT
+    KC_DIAG, KC_MISC, KC_IR_ADDCORR, KC_BETA0, KC_SOLVE2D, KC_COUNT
 };
 
 // Launch counter and optional CUDA-event timer per kernel class. Event pairs
@@ -355,6 +355,17 @@ void launch_in_dir(const Dims& g, const Phys& ph, const SolveIO<T, DIM>& io, int
 template <typename T, int DIM>
 void launch_in_update(const Dims& g, const SolveIO<T, DIM>& io, int cur, int first, RedBuf rb,
                       CGScalars* sc, cudaStream_t s);
+// The whole 2D solve in one launch of a thread-block cluster (pf_solve2d.cu).
+// solve2d_plan: false when the grid does not fit (use the kernels above).
+// b0, b1: the face coefficients of level 0, written (null: none are kept).
+struct S2Plan;
+void solve2d_prepare();
+template <typename T>
+bool solve2d_plan(const MGHier<T>& H, bool beta_global, S2Plan& P);
+template <typename T>
+cudaError_t launch_solve2d(const S2Plan& P, const Dims& g, const Phys& ph,
+                           const SolveIO<T, 2>& io, const MGHier<T>& H, T* b0, T* b1,
+                           CGScalars* sc, cudaStream_t s);
 void launch_sum(int n, const double* x, RedBuf rb, double* out, cudaStream_t s);
 // Sets the condition of a WHILE node of a captured solve (which = 0: inner CG
 // loop, 1: outer refinement loop) from the solve's device scalars.

@@ -977,13 +977,7 @@ k_ir_residual(Dims g, Phys ph, SolveIO<T, DIM> io, int first, RedBuf rb, CGScala
     if (grid_reduce<3>(v, mode, rb, tot) && threadIdx.x == 0) ir_finish(tot, first, sc);
 }
 
-// x += e (mixed path: x a double-float, hi plane and lo plane)
-__device__ __forceinline__ void df_acc(float& h, float& l, float e) {
-    const f2 s = two_sum(h, e);
-    const f2 r = two_sum(s.hi, __fadd_rn(s.lo, l));
-    h = r.hi;
-    l = r.lo;
-}
+// x += e
 template <typename T, int DIM>
 __global__ void __launch_bounds__(kThreads)
 k_ir_addcorr(Dims g, SolveIO<T, DIM> io, const CGScalars* sc) {
