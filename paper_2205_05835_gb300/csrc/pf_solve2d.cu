@@ -11,6 +11,7 @@
 // scalar leaves the cluster: every CTA forms the same totals from the same
 // partial sums in the same order.
 #include <mutex>
+#include <type_traits>
 
 #include "pf_device.cuh"
 #include "pf_solve2d.cuh"
@@ -19,10 +20,8 @@ namespace pf {
 
 namespace {
 
-constexpr int kS2Threads = 512;
 constexpr int kS2Warps = kS2Threads / 32;
-constexpr size_t kS2Smem = 220 * 1024;   // dynamic shared memory of a CTA
-constexpr int kTinyCells = 64;           // levels of one warp (of CTA 0)
+constexpr size_t kS2SmemMax = 227 * 1024;   // shared memory of a CTA
 
 template <typename T>
 struct S2Args {
@@ -74,42 +73,67 @@ __device__ __forceinline__ void merge(S2AccF& a, S2AccF b) {
 __device__ __forceinline__ void merge(S2AccD& a, S2AccD b) { a.s += b.s; }
 
 template <typename A>
-struct S2Red {
-    A warp[2][kS2Warps];
-    A part[2][2][kS2MaxCTAs];   // [buffer][value][CTA], written by every CTA of the cluster
+struct S2Red;
+template <>
+struct S2Red<S2AccF> {
+    S2AccF warp[2][kS2Warps];
+    S2AccF part[2][2][kS2MaxCTAs];   // [buffer][value][CTA], written by every CTA of the cluster
+};
+template <>
+struct S2Red<S2AccD> {
+    S2AccD all[2][kS2Threads];
+    S2AccD part[2][2][kS2MaxCTAs];
 };
 
-// K totals over the cluster, valid in warp 0 of every CTA. Contains a cluster
-// barrier, which also orders the phases before and after it. The partial sums
-// are pushed into every CTA's memory before that barrier, so nothing remote is
-// read after it.
+// K totals over the cluster, valid in lane 0 of warps 0 .. K - 1 of every CTA
+// (value k in warp k). Contains a cluster barrier, which also orders the phases
+// before and after it. The partial sums are pushed into every CTA's memory
+// before that barrier, so nothing remote is read after it.
+// Float pairs are summed by shuffles in every warp; float64 values go through
+// shared memory, so that one warp per value adds 16 of them per lane: a shuffle
+// tree in all 16 warps would issue five times the float64 instructions (each
+// occupies GB300's two-lane float64 pipe for 16 cycles).
 template <int K, typename A>
-__device__ __forceinline__ void cluster_totals(A (&v)[K], S2Red<A>& R, int C, int rank, int& buf) {
+__device__ __forceinline__ void cluster_totals(A (&v)[K], A& tot, S2Red<A>& R, int C, int rank,
+                                               int& buf) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if constexpr (sizeof(A) == sizeof(S2AccF) && !std::is_same<A, S2AccD>::value) {
 #pragma unroll
-    for (int k = 0; k < K; ++k)
+        for (int k = 0; k < K; ++k)
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) merge(v[k], shfl_acc(v[k], o));
-    if (lane == 0)
+            for (int o = 16; o > 0; o >>= 1) merge(v[k], shfl_acc(v[k], o));
+        if (lane == 0)
 #pragma unroll
-        for (int k = 0; k < K; ++k) R.warp[k][warp] = v[k];
-    __syncthreads();
-    if (warp == 0) {
+            for (int k = 0; k < K; ++k) R.warp[k][warp] = v[k];
+        __syncthreads();
+        if (warp < K) {
+            tot = R.warp[warp][lane & (kS2Warps - 1)];
 #pragma unroll
-        for (int k = 0; k < K; ++k) {
-            v[k] = R.warp[k][lane & (kS2Warps - 1)];
+            for (int o = kS2Warps / 2; o > 0; o >>= 1) merge(tot, shfl_acc(tot, o));
+        }
+    } else {
 #pragma unroll
-            for (int o = kS2Warps / 2; o > 0; o >>= 1) merge(v[k], shfl_acc(v[k], o));
-            if (lane < C) *cluster_map(&R.part[buf][k][rank], lane) = v[k];
+        for (int k = 0; k < K; ++k) R.all[k][threadIdx.x] = v[k];
+        __syncthreads();
+        if (warp < K) {
+            A s[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) s[j] = R.all[warp][lane + 32 * j];
+#pragma unroll
+            for (int j = 4; j < kS2Warps; ++j) merge(s[j & 3], R.all[warp][lane + 32 * j]);
+            merge(s[0], s[1]);
+            merge(s[2], s[3]);
+            merge(s[0], s[2]);
+            tot = s[0];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) merge(tot, shfl_acc(tot, o));
         }
     }
+    if (warp < K && lane < C) *cluster_map(&R.part[buf][warp][rank], lane) = tot;
     cluster_sync(C);
-    if (warp == 0) {
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            v[k] = R.part[buf][k][lane & (C - 1)];
-            for (int o = C >> 1; o > 0; o >>= 1) merge(v[k], shfl_acc(v[k], o));
-        }
+    if (warp < K) {
+        tot = R.part[buf][warp][lane & (C - 1)];
+        for (int o = C >> 1; o > 0; o >>= 1) merge(tot, shfl_acc(tot, o));
     }
     buf ^= 1;
 }
@@ -118,78 +142,46 @@ __device__ __forceinline__ void cluster_totals(A (&v)[K], S2Red<A>& R, int C, in
 template <typename T>
 struct S2Scal {
     T alpha, beta;
-    double rz, alpha_d;
-    double ff, rr, rr0_in, rr_in, eta2;
+    double rz, zq, pq;
+    double ff, rr, rr0_in, eta2;
     int done, idone, iters, it_in, outer, status, capped;
 };
 
-// Sweeps and transfers of the levels held by CTA 0: barriers of the whole CTA
-// above the tiny levels, of warp 0 within them.
+// The part of the V-cycle on the levels held by CTA 0 (the first one's right-
+// hand side and its sweep's start are in place).
 template <typename T>
-__device__ __forceinline__ void tiny_vcycle(S2View<T>* S, int l0, int lb, int pre, int post,
-                                            int bottom) {
-    const int t = threadIdx.x;   // < 32
-    for (int l = l0; l < lb; ++l) {
+__device__ __forceinline__ void single_vcycle(const S2View<T>* S, int lc, int ld, int pre,
+                                              int post, unsigned fused_levels, const T* M) {
+    const int t = threadIdx.x;
+    for (int l = lc; l < ld; ++l) {
         const int nc = s2_classes(S[l]);
         for (int s = 0; s < pre; ++s)
-            for (int k = 0; k < nc; ++k) {
-                s2_gs(S[l], k, s == 0 && k == 0, t, 32);
-                __syncwarp();
-            }
-        s2_restrict(S[l], S[l + 1], pre == 1, t, 32);
-        __syncwarp();
-    }
-    {
-        // bottom level (at most 3 x 3 cells): remove the mean, then sweep
-        const S2View<T>& B = S[lb];
-        const int n = B.nx * B.ny;
-        typename S2AccOf<T>::type a{};
-        for (int i = 0; i < n; ++i) a.add_prod(B.f[i], T(1));
-        const T mean = T(a.s) / T(n);
-        __syncwarp();
-        if (t < n) B.f[t] -= mean;
-        __syncwarp();
-        const int nc = s2_classes(B);
-        for (int s = 0; s < bottom; ++s)
-            for (int k = 0; k < nc; ++k) {
-                s2_gs(B, k, s == 0 && k == 0, t, 32);
-                __syncwarp();
-            }
-    }
-    for (int l = lb - 1; l >= l0; --l) {
-        s2_prolong(S[l], S[l + 1], t, 32);
-        __syncwarp();
-        const int nc = s2_classes(S[l]);
-        for (int s = 0; s < post; ++s)
-            for (int k = nc - 1; k >= 0; --k) {
-                s2_gs(S[l], k, false, t, 32);
-                __syncwarp();
-            }
-    }
-}
-template <typename T>
-__device__ __forceinline__ void single_vcycle(S2View<T>* S, int lc, int lt, int lb, int pre,
-                                              int post, int bottom) {
-    const int t = threadIdx.x, nt = kS2Threads;
-    for (int l = lc; l < lt; ++l) {
-        const int nc = s2_classes(S[l]);
-        for (int s = 0; s < pre; ++s)
-            for (int k = 0; k < nc; ++k) {
-                s2_gs(S[l], k, s == 0 && k == 0, t, nt);
+            for (int k = s == 0 ? 1 : 0; k < nc; ++k) {
+                s2_gs(S[l], k, t);
                 __syncthreads();
             }
-        s2_restrict(S[l], S[l + 1], pre == 1, t, nt);
+        s2_restrict(S[l], S[l + 1], pre == 1, t);
         __syncthreads();
     }
-    if (t < 32) tiny_vcycle(S, lt, lb, pre, post, bottom);
-    __syncthreads();
-    for (int l = lt - 1; l >= lc; --l) {
-        s2_prolong(S[l], S[l + 1], t, nt);
+    {
+        const S2View<T>& B = S[ld];
+        const int n = B.nx * B.ny;
+        T x = s2_dense_part(M, B.f, n, t);
+        x += __shfl_xor_sync(0xffffffffu, x, 1);
+        x += __shfl_xor_sync(0xffffffffu, x, 2);
+        x += __shfl_xor_sync(0xffffffffu, x, 4);
+        if ((t & 7) == 0 && (t >> 3) < n) B.x[t >> 3] = x;
+        __syncthreads();
+    }
+    for (int l = ld - 1; l >= lc; --l) {
+        const bool fused = (fused_levels >> l) & 1;
+        if (fused) s2_prolong_gs(S[l], S[l + 1], t);
+        else s2_prolong(S[l], S[l + 1], t);
         __syncthreads();
         const int nc = s2_classes(S[l]);
         for (int s = 0; s < post; ++s)
-            for (int k = nc - 1; k >= 0; --k) {
-                s2_gs(S[l], k, false, t, nt);
+            for (int k = nc - 1 - (fused && s == 0 ? 1 : 0); k >= 0; --k) {
+                s2_gs(S[l], k, t);
                 __syncthreads();
             }
     }
@@ -201,7 +193,7 @@ __device__ __forceinline__ void single_vcycle(S2View<T>* S, int lc, int lt, int 
 template <typename T>
 __device__ __forceinline__ void s2_residual(const S2Args<T>& a, const S2View<T>& L, double mb,
                                             bool first, T& ff, T& rr) {
-    const int nx = L.nx, n = L.rows * nx;
+    const int nx = L.nx;
     const bool pos = a.io.sign > 0.0;
     const int N = a.g.ncell;
     if constexpr (sizeof(T) == sizeof(float)) {
@@ -212,8 +204,8 @@ __device__ __forceinline__ void s2_residual(const S2Args<T>& a, const S2View<T>&
         const f2 mdf = df_neg(df_of(mb));
         const f2 ih2 = df_of(a.g.ih2);
         const float h2 = float(a.g.h * a.g.h);
-        for (int q = threadIdx.x; q < n; q += kS2Threads) {
-            const int r = s2_div(q, L.inv_nx), i = q - r * nx, j = L.j0 + r;
+        s2_cells(nx, L.rows, L.lf, threadIdx.x, [&](int r, int i) {
+            const int q = r * nx + i, j = L.j0 + r;
             const int idx = j * nx + i;
             f2 f = df_add(f2{bh[idx], bl[idx]}, mdf);
             if (!pos) f = df_neg(f);
@@ -232,17 +224,18 @@ __device__ __forceinline__ void s2_residual(const S2Args<T>& a, const S2View<T>&
             const f2 rv = df_add(f, df_neg(ax));
             const float rt = __fadd_rn(rv.hi, rv.lo);
             L.f[q] = rt * h2;
+            s2_start(L, i, j, q, rt * h2);
             if (first) {
                 const float ft = __fadd_rn(f.hi, f.lo);
                 ff += ft * ft;
             }
             rr += rt * rt;
-        }
+        });
     } else {
         const double h2 = a.g.h * a.g.h;
         const double* x = a.io.x;
-        for (int q = threadIdx.x; q < n; q += kS2Threads) {
-            const int r = s2_div(q, L.inv_nx), i = q - r * nx, j = L.j0 + r;
+        s2_cells(nx, L.rows, L.lf, threadIdx.x, [&](int r, int i) {
+            const int q = r * nx + i, j = L.j0 + r;
             const int idx = j * nx + i;
             const double f = pos ? a.io.b[idx] - mb : mb - a.io.b[idx];
             const int m0 = i == 0 ? idx + nx - 1 : idx - 1, m1 = i == nx - 1 ? idx - i : idx + 1;
@@ -255,9 +248,10 @@ __device__ __forceinline__ void s2_residual(const S2Args<T>& a, const S2View<T>&
             ax += (r == L.rows - 1 ? L.w1p[i] : L.w1[q + nx]) * (xc - __ldcg(x + m3));
             const double rv = f - ax * a.g.ih2;
             L.f[q] = rv * h2;
+            s2_start(L, i, j, q, rv * h2);
             if (first) ff += f * f;
             rr += rv * rv;
-        }
+        });
     }
 }
 
@@ -271,9 +265,11 @@ __global__ void __launch_bounds__(kS2Threads, 1) k_solve2d(const __grid_constant
     __shared__ S2Red<A> R;
     __shared__ S2Scal<T> sc;
     __shared__ T *vp, *vpm, *vpp, *vq, *ve;
+    __shared__ T colrow[2 * kS2ColRow];
     const S2Plan& P = a.P;
     const int C = P.C, rank = cluster_rank(), tid = threadIdx.x;
-    const int lc = P.lc, lb = P.nlev - 1;
+    const int lc = P.lc, ld = P.ld;
+    T* M = sm + P.om;
 
     // ---- this CTA's views ----
     if (tid <= lc) {
@@ -291,7 +287,7 @@ __global__ void __launch_bounds__(kS2Threads, 1) k_solve2d(const __grid_constant
             v.f = b + L.of + j0 * L.nx;
             v.w0 = b + L.ow0 + j0 * L.nx;
             v.w1 = b + L.ow1 + j0 * L.nx;
-            v.di = nullptr;
+            v.di = b + L.od + j0 * L.nx;
             v.xm = b + L.ox + jm * L.nx;
             v.xp = b + L.ox + jp * L.nx;
             v.w1p = b + L.ow1 + jp * L.nx;
@@ -314,13 +310,13 @@ __global__ void __launch_bounds__(kS2Threads, 1) k_solve2d(const __grid_constant
             v.w1p = dn(L.ow1, a.gw1[gl]);
             if (l == 0) {
                 vp = own(P.op, a.gp);
-                vpm = up(P.op, a.gp);
-                vpp = dn(P.op, a.gp);
                 vq = own(P.oq, a.gq);
                 ve = own(P.oe, a.ge);
+                vpm = up(P.op, a.gp);
+                vpp = dn(P.op, a.gp);
             }
         }
-    } else if (tid >= 32 && tid - 32 + lc <= lb) {
+    } else if (tid >= 32 && tid - 32 + lc <= ld) {
         const int l = tid - 32 + lc;
         const S2Lev& L = P.lev[l];
         S2View<T>& v = S[l];
@@ -334,16 +330,14 @@ __global__ void __launch_bounds__(kS2Threads, 1) k_solve2d(const __grid_constant
         v.xp = v.x;
         v.w1p = v.w1;
     }
-    int lt = lb;   // first level of one warp
-    while (lt > lc && P.lev[lt - 1].nx * P.lev[lt - 1].ny <= kTinyCells) --lt;
     __syncthreads();
     const S2View<T>& L0 = V[0];
 
     // ---- face coefficients of level 0 ----
     {
-        const int nx = L0.nx, n = L0.rows * nx;
-        for (int q = tid; q < n; q += kS2Threads) {
-            const int r = s2_div(q, L0.inv_nx), i = q - r * nx, j = L0.j0 + r;
+        const int nx = L0.nx;
+        s2_cells(nx, L0.rows, L0.lf, tid, [&](int r, int i) {
+            const int q = r * nx + i, j = L0.j0 + r;
             const int idx = j * nx + i;
             const int m0 = i == 0 ? idx + nx - 1 : idx - 1;
             const int m2 = j == 0 ? idx + (L0.ny - 1) * nx : idx - nx;
@@ -365,22 +359,45 @@ __global__ void __launch_bounds__(kS2Threads, 1) k_solve2d(const __grid_constant
                 a.b0[idx] = w0;
                 a.b1[idx] = w1;
             }
-        }
+        });
     }
     cluster_sync(C);
     // ---- coarse coefficients (a coarse row's children are the CTA's own) ----
     for (int l = 0; l < lc; ++l) {
-        s2_coarsen(V[l], V[l + 1], tid, kS2Threads);
+        s2_coarsen(V[l], V[l + 1], tid);
         __syncthreads();
     }
     cluster_sync(C);
-    for (int l = 0; l < lc; ++l) s2_invdiag(V[l], tid, kS2Threads);
-    if (rank == 0)
-        for (int l = lc; l <= lb; ++l) {
-            s2_invdiag(S[l], tid, kS2Threads);
-            if (l < lb) s2_coarsen(S[l], S[l + 1], tid, kS2Threads);
+    for (int l = 0; l < lc; ++l) s2_invdiag(V[l], tid);
+    if (rank == 0) {
+        for (int l = lc; l <= ld; ++l) {
+            s2_invdiag(S[l], tid);
+            if (l < ld) s2_coarsen(S[l], S[l + 1], tid);
             __syncthreads();
         }
+        const int n = S[ld].nx * S[ld].ny;
+        s2_dense_build(S[ld], M, tid);
+        __syncthreads();
+        s2_dense_fill(S[ld], M, tid);
+        __syncthreads();
+        T m[8];
+        s2_gj_move(m, M, n, false, tid);
+        s2_gj_publish(m, n, 0, colrow, tid);
+        __syncthreads();
+        for (int k = 0; k < n; ++k) {
+            s2_gj_step(m, n, k, colrow + (k & 1) * kS2ColRow, tid);
+            s2_gj_publish(m, n, k + 1, colrow + ((k + 1) & 1) * kS2ColRow, tid);
+            __syncthreads();
+        }
+        s2_gj_move(m, M, n, true, tid);
+        __syncthreads();
+        for (int k = 0; k < 3; ++k) {
+            s2_dense_means(S[ld], M, n, k, colrow, tid);
+            __syncthreads();
+        }
+        s2_dense_project(M, n, colrow, tid);
+    }
+    __syncthreads();
 
     // ---- iterative refinement ----
     const double mb = a.sc->mean_b, rtol2 = a.sc->rtol2, eta2_min = a.sc->eta2_min;
@@ -393,18 +410,18 @@ __global__ void __launch_bounds__(kS2Threads, 1) k_solve2d(const __grid_constant
         {
             T ff = T(0), rr = T(0);
             s2_residual(a, L0, mb, first_res, ff, rr);
-            A v[2] = {acc_of(ff), acc_of(rr)};
-            cluster_totals<2>(v, R, C, rank, buf);
+            A v[2] = {acc_of(ff), acc_of(rr)}, tot{};
+            cluster_totals<2>(v, tot, R, C, rank, buf);
+            if (tid == 32) sc.rr = tot.value();
+            __syncthreads();
             if (tid == 0) {
                 // as ir_finish
                 if (first_res) {
-                    sc.ff = v[0].value();
+                    sc.ff = tot.value();
                     sc.iters = sc.capped = sc.done = sc.status = 0;
                 }
-                const double rrv = v[1].value();
-                sc.rr = rrv;
+                const double rrv = sc.rr;
                 sc.rr0_in = rrv * h4;
-                sc.rr_in = sc.rz = 0.0;
                 sc.outer = outer + 1;
                 sc.idone = 0;
                 if (!(rrv == rrv)) {
@@ -425,62 +442,65 @@ __global__ void __launch_bounds__(kS2Threads, 1) k_solve2d(const __grid_constant
         if (sc.done || outer == 64) break;
         for (int it = 0;; ++it) {
             const bool first = it == 0;
-            // V-cycle, down
+            // V-cycle, down (each sweep's first class from zero came with f)
             for (int l = 0; l < lc; ++l) {
                 const S2View<T>& L = V[l];
                 const int nc = s2_classes(L);
                 for (int s = 0; s < P.pre; ++s)
-                    for (int k = 0; k < nc; ++k) {
-                        s2_gs(L, k, s == 0 && k == 0, tid, kS2Threads);
+                    for (int k = s == 0 ? 1 : 0; k < nc; ++k) {
+                        s2_gs(L, k, tid);
                         cluster_sync(C);
                     }
-                s2_restrict(L, V[l + 1], P.pre == 1, tid, kS2Threads);
-                if (l + 1 < lc) __syncthreads();
-                else cluster_sync(C);
+                s2_restrict(L, V[l + 1], P.pre == 1, tid);
+                cluster_sync(C);
             }
-            if (rank == 0)
-                single_vcycle(S, lc, lt, lb, P.pre, P.post, P.bottom_sweeps);
+            if (rank == 0) single_vcycle(S, lc, ld, P.pre, P.post, P.fused, M);
             cluster_sync(C);
             // up
-            A d[2] = {A{}, A{}};
+            A d[2] = {A{}, A{}}, tot{};
             for (int l = lc - 1; l >= 0; --l) {
                 const S2View<T>& L = V[l];
-                s2_prolong(L, V[l + 1], tid, kS2Threads);
+                // one phase less where a thread has few cells (the interpolation is
+                // then formed four times)
+                const bool fused = (P.fused >> l) & 1;
+                if (fused) s2_prolong_gs(L, V[l + 1], tid);
+                else s2_prolong(L, V[l + 1], tid);
                 cluster_sync(C);
                 const int nc = s2_classes(L);
                 for (int s = 0; s < P.post; ++s)
-                    for (int k = nc - 1; k >= 0; --k) {
+                    for (int k = nc - 1 - (fused && s == 0 ? 1 : 0); k >= 0; --k) {
                         if (l == 0 && s == P.post - 1 && k == 0) {
-                            s2_gs_dots(L, vq, first, d[0], d[1], tid, kS2Threads);
+                            s2_gs_dots(L, vq, first, d[0], d[1], tid);
                         } else {
-                            s2_gs(L, k, false, tid, kS2Threads);
+                            s2_gs(L, k, tid);
                             cluster_sync(C);
                         }
                     }
             }
-            cluster_totals<2>(d, R, C, rank, buf);
+            // flexible CG: beta = -z.q / (p.q) of the last direction (Polak-Ribiere:
+            // alpha q is the last change of r)
+            cluster_totals<2>(d, tot, R, C, rank, buf);
+            if (tid == 32) sc.zq = tot.value();
+            __syncthreads();
             if (tid == 0) {
-                const double rz = d[0].value();
-                sc.beta = first ? T(0) : T(-sc.alpha_d * d[1].value() / sc.rz);
-                sc.rz = rz;
+                sc.rz = tot.value();
+                sc.beta = first ? T(0) : T(-sc.zq / sc.pq);
             }
             __syncthreads();
-            s2_direction(L0, vp, sc.beta, first, tid, kS2Threads);
+            s2_direction(L0, vp, sc.beta, first, tid);
             cluster_sync(C);
             A pq[1] = {A{}};
-            s2_apply(L0, vp, vpm, vpp, vq, pq[0], tid, kS2Threads);
-            cluster_totals<1>(pq, R, C, rank, buf);
+            s2_apply(L0, vp, vpm, vpp, vq, pq[0], tid);
+            cluster_totals<1>(pq, tot, R, C, rank, buf);
             if (tid == 0) {
-                const double v = pq[0].value();
-                sc.alpha_d = v != 0.0 ? sc.rz / v : 0.0;
-                sc.alpha = T(sc.alpha_d);
+                sc.pq = tot.value();
+                sc.alpha = T(sc.pq != 0.0 ? sc.rz / sc.pq : 0.0);
             }
             __syncthreads();
-            A rr[1] = {acc_of(s2_update(L0, vp, vq, ve, sc.alpha, first, tid, kS2Threads))};
-            cluster_totals<1>(rr, R, C, rank, buf);
+            A rr[1] = {acc_of(s2_update(L0, vp, vq, ve, sc.alpha, first, tid))};
+            cluster_totals<1>(rr, tot, R, C, rank, buf);
             if (tid == 0) {
-                const double v = rr[0].value();
-                sc.rr_in = v;
+                const double v = tot.value();
                 sc.iters += 1;
                 if (!(v == v) || v <= sc.eta2 * sc.rr0_in) {
                     sc.idone = 1;
@@ -519,11 +539,40 @@ __global__ void __launch_bounds__(kS2Threads, 1) k_solve2d(const __grid_constant
     cluster_sync(C);   // no CTA leaves while another may read its memory
 }
 
-// Levels of at most this many cells go to CTA 0: about the size where a phase
-// over the cluster costs what one CTA's phase does (the float64 pipe makes that
-// smaller for float64).
-template <typename T> constexpr int kSingleCells = sizeof(T) == 4 ? 1024 : 256;
-template <typename T> constexpr int kCtaCells = sizeof(T) == 4 ? 512 : 256;
+// Largest strip (cells of level 0 per CTA) the cluster takes. Beyond it the
+// kernels on the whole chip are faster: a mixed step of 640^2 takes 5.3 ms
+// here and 7.3 ms there, of 768^2 9.5 and 6.2 ms; a float64 one of 512^2 11.3
+// and 13.8 ms (larger ones do not fit).
+template <typename T> constexpr int kMaxCtaCells = sizeof(T) == 4 ? 27000 : 16500;
+
+// dynamic shared memory left beside the kernel's static arrays
+template <typename T>
+size_t dynamic_smem() {
+    cudaFuncAttributes at;
+    if (cudaFuncGetAttributes(&at, k_solve2d<T>) != cudaSuccess) return 0;
+    return kS2SmemMax - ((at.sharedSizeBytes + 1023) & ~(size_t)1023);
+}
+
+template <typename T>
+S2Limits limits(int max_cluster) {
+    // Cycles measured at 64^2 .. 256^2: a phase of a cluster costs about 900
+    // beside its cells, one of a CTA 400. The inverse of 64 cells costs about
+    // 20k cycles a solve in float32, a float64 one of 16 cells as much. The
+    // fused interpolation has 31 instructions a cell instead of 4, too many for
+    // the float64 pipe.
+    const bool f32 = sizeof(T) == 4;
+    S2Limits m;
+    m.max_cluster = max_cluster;
+    m.dense_cells = f32 ? 64 : 16;
+    m.fused_cells = f32 ? 2048 : 0;
+    m.cta_cells = kMaxCtaCells<T>;
+    m.cell = f32 ? 8.f : 28.f;
+    m.single_cell = f32 ? 5.f : 13.f;
+    m.phase = 900.f;
+    m.cta_phase = 400.f;
+    m.smem_bytes = dynamic_smem<T>();
+    return m;
+}
 
 template <typename T>
 int max_cluster() {
@@ -531,13 +580,13 @@ int max_cluster() {
     static int best = 0;
     std::call_once(once, [] {
         cudaFuncSetAttribute(k_solve2d<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)kS2Smem);
+                             (int)dynamic_smem<T>());
         cudaFuncSetAttribute(k_solve2d<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         for (int c = kS2MaxCTAs; c >= 1 && best == 0; c >>= 1) {
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3(c);
             cfg.blockDim = dim3(kS2Threads);
-            cfg.dynamicSmemBytes = kS2Smem;
+            cfg.dynamicSmemBytes = dynamic_smem<T>();
             cudaLaunchAttribute at[1];
             at[0].id = cudaLaunchAttributeClusterDimension;
             at[0].val.clusterDim.x = c;
@@ -563,7 +612,7 @@ void solve2d_prepare() {
 template <typename T>
 bool solve2d_plan(const MGHier<T>& H, bool beta_global, S2Plan& P) {
     const int mc = max_cluster<T>();
-    return mc > 0 && s2_plan<T>(H, kSingleCells<T>, kCtaCells<T>, mc, kS2Smem, beta_global, P);
+    return mc > 0 && s2_plan<T>(H, limits<T>(mc), beta_global, P);
 }
 
 template <typename T>

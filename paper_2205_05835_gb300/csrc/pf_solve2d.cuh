@@ -9,6 +9,8 @@
 
 #include <math.h>
 
+#include <type_traits>
+
 #include "pf_internal.h"
 
 #ifdef __CUDACC__
@@ -35,12 +37,18 @@ struct S2Lev {
 struct S2Plan {
     int C;             // CTAs of the cluster
     int lc;            // first level held by CTA 0 alone
-    int nlev;
-    int pre, post, bottom_sweeps;
+    int ld;            // dense level: solved by its inverse (lc <= ld)
+    int pre, post;
     int op, oq, oe;    // offsets of p, q, e (-1: workspace)
+    int om;            // the dense level's inverse, padded rows of s2_pad(cells)
     int elems;         // dynamic shared memory, elements
+    unsigned fused;    // bit l: s2_prolong_gs on level l (the same in every CTA)
     S2Lev lev[kMaxLevels];
 };
+
+// Row pitch of the dense inverse: 8 segments of a row are read at once, pitch 8
+// mod 32 puts four rows of them on different banks (4-byte elements).
+PF_HD int s2_pad(int n) { return ((n + 31) & ~31) + 8; }
 
 // First row of CTA c's strip on level l <= lc (c = C: the level's end). Strips
 // are multiples of the coarser levels' strips, so a coarse row's children and
@@ -49,19 +57,35 @@ PF_HD int s2_row(const S2Plan& P, int l, int c) {
     if (c >= P.C) return P.lev[l].ny;
     return ((P.lev[P.lc].ny * c) / P.C) << (P.lc - l);
 }
+inline int s2_max_rows(const S2Plan& P, int l) {
+    if (l >= P.lc) return P.lev[l].ny;
+    int m = 0;
+    for (int c = 0; c < P.C; ++c) {
+        const int r = s2_row(P, l, c + 1) - s2_row(P, l, c);
+        if (r > m) m = r;
+    }
+    return m;
+}
+
+// What decides the plan: the largest cluster, the dense level's cells, the
+// strip's cells up to which the interpolation joins the first post class, the
+// dynamic shared memory, and a cost model of an iteration in cycles: per cell
+// of the largest strip, per cell of the levels of CTA 0, per phase of a cluster
+// and of a CTA.
+struct S2Limits {
+    int max_cluster, dense_cells, fused_cells, cta_cells;
+    float cell, single_cell, phase, cta_phase;
+    size_t smem_bytes;
+};
 
 // Fits the solve of a hierarchy into a cluster's shared memory: false when it
-// does not (too large a grid). single_cells: levels of at most this many cells
-// go to CTA 0; cta_cells: cells of level 0 per CTA below which the cluster
-// shrinks; beta_global: the face coefficients also exist in the workspace.
+// does not (too large a grid: more than cta_cells cells a CTA). beta_global:
+// the face coefficients also exist in the workspace.
 template <typename T>
-inline bool s2_plan(const MGHier<T>& H, int single_cells, int cta_cells, int max_cluster,
-                    size_t smem_bytes, bool beta_global, S2Plan& P) {
+inline bool s2_plan(const MGHier<T>& H, const S2Limits& lim, bool beta_global, S2Plan& P) {
     if (H.nlev < 2 || H.lev[0].g.nz != 1) return false;
-    P.nlev = H.nlev;
     P.pre = H.pre;
     P.post = H.post;
-    P.bottom_sweeps = H.coarse_sweeps;
     for (int l = 0; l < H.nlev; ++l) {
         S2Lev& L = P.lev[l];
         L.nx = H.lev[l].g.nx;
@@ -71,53 +95,64 @@ inline bool s2_plan(const MGHier<T>& H, int single_cells, int cta_cells, int max
         L.qx = H.lev[l].lastw[0];
         L.qy = H.lev[l].lastw[1];
     }
+    auto cells = [&](int l) { return P.lev[l].nx * P.lev[l].ny; };
     // the bottom must be small (a hierarchy of even halvings alone may not be)
-    if (P.lev[P.nlev - 1].nx > 3 || P.lev[P.nlev - 1].ny > 3) return false;
-    P.lc = 1;
-    while (P.lc < P.nlev - 1 && P.lc < kS2MaxCluster - 1 &&
-           P.lev[P.lc].nx * P.lev[P.lc].ny > single_cells)
-        ++P.lc;
-    P.C = 1;
-    while (2 * P.C <= max_cluster && 2 * P.C <= kS2MaxCTAs && P.lev[P.lc].ny >= 2 * P.C &&
-           (long long)P.lev[0].nx * P.lev[0].ny >= (long long)2 * P.C * cta_cells)
-        P.C *= 2;
-    long long off = 0;
-    const long long cap = (long long)(smem_bytes / sizeof(T));
-    auto take = [&](long long n) {
-        const int o = (int)off;
-        off += (n + 3) & ~3LL;
-        return o;
-    };
-    auto fits = [&](int* slot, long long n) {
-        *slot = -1;
-        if (off + n + 3 <= cap) *slot = take(n);
-        return *slot >= 0;
-    };
-    for (int l = P.nlev - 1; l >= 0; --l) {
-        S2Lev& L = P.lev[l];
-        long long rows = L.ny;
-        if (l < P.lc) {
-            rows = 0;
-            for (int c = 0; c < P.C; ++c) {
-                const int r = s2_row(P, l, c + 1) - s2_row(P, l, c);
-                if (r > rows) rows = r;
+    if (cells(H.nlev - 1) > lim.dense_cells) return false;
+    // the split with the least modelled cost: more cluster levels make the
+    // strips coarser (unequal), fewer leave more to CTA 0
+    float best = -1.f;
+    S2Plan Q = P;
+    for (int lc = 1; lc < H.nlev && lc < kS2MaxCluster; ++lc)
+        for (int C = 1; C <= lim.max_cluster && C <= kS2MaxCTAs && C <= P.lev[lc].ny; C *= 2) {
+            Q.lc = lc;
+            Q.C = C;
+            float c = 5.f * float(lc) * (C == 1 ? lim.cta_phase : lim.phase);
+            for (int l = 0; l < lc; ++l)
+                c += (l == 0 ? lim.cell : lim.single_cell) * float(s2_max_rows(Q, l) * P.lev[l].nx);
+            for (int l = lc; l < H.nlev && cells(l) > lim.dense_cells; ++l)
+                c += lim.single_cell * float(cells(l)) + 5.f * lim.cta_phase;
+            if (best < 0.f || c < best) {
+                best = c;
+                P.lc = lc;
+                P.C = C;
             }
         }
-        const long long n = rows * L.nx;
-        if (l >= 1) {
-            // coarse levels in shared memory; level 1, if it is a cluster level,
-            // may leave what has a place in the workspace there
-            const bool must = l >= P.lc || l >= 2;
-            int* slots[5] = {&L.od, &L.ox, &L.ow0, &L.ow1, &L.of};
-            for (int s = 0; s < 5; ++s)
-                if (!fits(slots[s], n) && (must || s == 0)) return false;
-        } else {
-            // level 0: the arrays that neighbours read and every phase touches first
-            int* slots[8] = {&L.ox, &L.ow0, &L.ow1, &L.od, &P.op, &L.of, &P.oq, &P.oe};
-            for (int s = 0; s < 8; ++s) fits(slots[s], n);
-        }
+    if (s2_max_rows(P, 0) * P.lev[0].nx > lim.cta_cells) return false;
+    P.ld = P.lc;
+    while (cells(P.ld) > lim.dense_cells) ++P.ld;
+    long long off = 0;
+    const long long cap = (long long)(lim.smem_bytes / sizeof(T));
+    auto fits = [&](int* slot, long long n) {
+        *slot = -1;
+        if (off + n + 3 > cap) return false;
+        *slot = (int)off;
+        off += (n + 3) & ~3LL;
+        return true;
+    };
+    if (!fits(&P.om, (long long)cells(P.ld) * s2_pad(cells(P.ld)))) return false;
+    for (int l = P.ld; l >= 1; --l) {
+        // coarse levels in shared memory; level 1, if it is a cluster level,
+        // may leave what has a place in the workspace there
+        S2Lev& L = P.lev[l];
+        const long long n = (long long)s2_max_rows(P, l) * L.nx;
+        const bool must = l >= P.lc || l >= 2;
+        int* slots[5] = {&L.od, &L.ox, &L.ow0, &L.ow1, &L.of};
+        for (int s = 0; s < 5; ++s)
+            if (!fits(slots[s], n) && (must || s == 0)) return false;
     }
-    if (!beta_global && (P.lev[0].ow0 < 0 || P.lev[0].ow1 < 0)) return false;
+    // level 0, in the order of use
+    S2Lev& L = P.lev[0];
+    const long long n0 = (long long)s2_max_rows(P, 0) * L.nx;
+    int* slots[8] = {&L.ox, &L.ow0, &L.ow1, &L.of, &L.od, &P.op, &P.oq, &P.oe};
+    for (int s = 0; s < 8; ++s) fits(slots[s], n0);
+    P.fused = 0;
+    for (int l = 0; l < P.ld; ++l) {
+        const S2Lev &F = P.lev[l], &N = P.lev[l + 1];
+        const bool even = F.nx > 1 && F.ny > 1 && F.nx % 2 == 0 && F.ny % 2 == 0;
+        if (even && N.qx == 1.f && N.qy == 1.f && s2_max_rows(P, l) * F.nx <= lim.fused_cells)
+            P.fused |= 1u << l;
+    }
+    if (!beta_global && (L.ow0 < 0 || L.ow1 < 0)) return false;
     P.elems = (int)off;
     return true;
 }
@@ -130,12 +165,19 @@ struct S2View {
     int nx, ny, j0, rows;
     int cfx, cfy;
     int seams;          // odd axes: bit 0 x, bit 1 y; bit 2: an axis of one cell
+    int lf, lh;         // log2 of the threads along a row: cells, pairs of cells
     float qx, qy;
-    float inv_nx, inv_nhx;
     T *x, *f, *w0, *w1, *di;
     T *xm, *xp, *w1p;
 };
 
+constexpr int kS2Threads = 512;
+
+PF_HD int s2_log2(int n) {   // threads along a row of n items
+    int l = 0;
+    while ((1 << l) < n && (2 << l) <= kS2Threads) ++l;
+    return l;
+}
 template <typename T>
 PF_HD void s2_view_sizes(S2View<T>& v, const S2Lev& L, int j0, int rows) {
     v.nx = L.nx;
@@ -145,17 +187,42 @@ PF_HD void s2_view_sizes(S2View<T>& v, const S2Lev& L, int j0, int rows) {
     v.cfx = L.cfx;
     v.cfy = L.cfy;
     v.seams = (L.nx > 1 ? (L.nx & 1) : 4) | (L.ny > 1 ? 2 * (L.ny & 1) : 4);
+    v.lf = s2_log2(L.nx);
+    v.lh = s2_log2((L.nx + 1) >> 1);
     v.qx = L.qx;
     v.qy = L.qy;
-    v.inv_nx = 1.0f / float(L.nx);
-    v.inv_nhx = 1.0f / float((L.nx + 1) >> 1);
 }
 template <typename T>
 PF_HD int s2_classes(const S2View<T>& L) { return 2 + 2 * ((L.seams & 1) + ((L.seams >> 1) & 1)); }
 
-// q / n for q < 2^22 with inv = 1 / n rounded to float: q + 1/2 over n lies at
-// least 1/(2n) from an integer and the two roundings move it by less.
-PF_HD int s2_div(int q, float inv) { return int((float(q) + 0.5f) * inv); }
+// Loops of a CTA's threads over its cells (f(r, i)) or pairs (2m, 2m + 1) of
+// cells of a row (f(r, m)): powers of two of threads along a row, so no thread
+// divides by the level's size.
+template <typename F>
+PF_HD void s2_cells(int n, int rows, int lw, int t, F f) {
+    const int i0 = t & ((1 << lw) - 1);
+    for (int r = t >> lw; r < rows; r += kS2Threads >> lw)
+        for (int i = i0; i < n; i += 1 << lw) f(r, i);
+}
+
+// The same for val(r, i), which only reads, and put(r, i, value): a thread with
+// several rows forms two rows' values before it stores the first, so that their
+// loads overlap (a store between them would order them). More rows at once, or
+// predicated ones, slowed the many phases with one row a thread by a quarter.
+template <typename V, typename F, typename G>
+PF_HD void s2_map(int n, int rows, int lw, int t, F val, G put) {
+    const int i0 = t & ((1 << lw) - 1), dr = kS2Threads >> lw;
+    int r = t >> lw;
+    if (!std::is_same<V, double>::value && sizeof(V) <= 8)   // (float64 phases wait for the pipe)
+        for (; r + dr < rows; r += 2 * dr)
+            for (int i = i0; i < n; i += 1 << lw) {
+                const V a = val(r, i), b = val(r + dr, i);
+                put(r, i, a);
+                put(r + dr, i, b);
+            }
+    for (; r < rows; r += dr)
+        for (int i = i0; i < n; i += 1 << lw) put(r, i, val(r, i));
+}
 
 PF_HD float s2_rcp(float a) {
 #ifdef __CUDA_ARCH__
@@ -166,43 +233,60 @@ PF_HD float s2_rcp(float a) {
 }
 PF_HD double s2_rcp(double a) { return 1.0 / a; }
 
-// sum of the four face coefficients times the neighbours, and of the coefficients
+// The four neighbours of a cell of the strip: offsets along the row, and the
+// rows above and below (chosen before the load, so the loads of a cell issue
+// together).
 template <typename T>
-PF_HD T s2_off(const S2View<T>& L, int r, int i, int idx) {
+struct S2Nb {
+    int il, ir;
+    const T *xu, *xd, *wd;
+};
+template <typename T>
+PF_HD S2Nb<T> s2_nb(const S2View<T>& L, int r, int i, int idx) {
     const int nx = L.nx;
-    const int il = i == 0 ? idx + nx - 1 : idx - 1;
-    const int ir = i == nx - 1 ? idx - i : idx + 1;
+    S2Nb<T> n;
+    n.il = i == 0 ? idx + nx - 1 : idx - 1;
+    n.ir = i == nx - 1 ? idx - i : idx + 1;
     const bool last = r == L.rows - 1;
-    const T xu = r == 0 ? L.xm[i] : L.x[idx - nx];
-    const T xd = last ? L.xp[i] : L.x[idx + nx];
-    const T wd = last ? L.w1p[i] : L.w1[idx + nx];
-    return L.w0[idx] * L.x[il] + L.w0[ir] * L.x[ir] + L.w1[idx] * xu + wd * xd;
+    n.xu = r == 0 ? L.xm + i : L.x + (idx - nx);
+    n.xd = last ? L.xp + i : L.x + (idx + nx);
+    n.wd = last ? L.w1p + i : L.w1 + (idx + nx);
+    return n;
+}
+// a plus the sum of the four face coefficients times the neighbours; the sum of
+// the coefficients
+template <typename T>
+PF_HD T s2_off(const S2View<T>& L, int r, int i, int idx, T a) {
+    const S2Nb<T> n = s2_nb(L, r, i, idx);
+    const T wl = L.w0[idx], wr = L.w0[n.ir], wu = L.w1[idx], wd = *n.wd;
+    const T xl = L.x[n.il], xr = L.x[n.ir], xu = *n.xu, xd = *n.xd;
+    // (one chain of multiply-adds: a float64 one takes a warp 63 cycles alone and
+    // 19 cycles of the SM, so their number counts, not their dependence)
+    a += wl * xl;
+    a += wr * xr;
+    a += wu * xu;
+    return a + wd * xd;
 }
 template <typename T>
 PF_HD T s2_diag(const S2View<T>& L, int r, int i, int idx) {
-    const int ir = i == L.nx - 1 ? idx - i : idx + 1;
-    const T wd = r == L.rows - 1 ? L.w1p[i] : L.w1[idx + L.nx];
-    return (L.w0[idx] + L.w0[ir]) + (L.w1[idx] + wd);
+    const S2Nb<T> n = s2_nb(L, r, i, idx);
+    return (L.w0[idx] + L.w0[n.ir]) + (L.w1[idx] + *n.wd);
 }
 
 // 1 / diagonal of the strip
 template <typename T>
-PF_HD void s2_invdiag(const S2View<T>& L, int t, int nt) {
-    const int n = L.rows * L.nx;
-    for (int q = t; q < n; q += nt) {
-        const int r = s2_div(q, L.inv_nx);
-        L.di[q] = s2_rcp(s2_diag(L, r, q - r * L.nx, q));
-    }
+PF_HD void s2_invdiag(const S2View<T>& L, int t) {
+    s2_cells(L.nx, L.rows, L.lf, t, [&](int r, int i) {
+        const int q = r * L.nx + i;
+        L.di[q] = s2_rcp(s2_diag(L, r, i, q));
+    });
 }
 
 // Face coefficients of the strip of the next level (see k_coarsen_beta).
 template <typename T>
-PF_HD void s2_coarsen(const S2View<T>& F, const S2View<T>& C, int t, int nt) {
-    const int n = C.rows * C.nx;
-    const int vol = F.cfx * F.cfy;
-    for (int q = t; q < n; q += nt) {
-        const int R = s2_div(q, C.inv_nx);
-        const int I = q - R * C.nx, J = C.j0 + R;
+PF_HD void s2_coarsen(const S2View<T>& F, const S2View<T>& C, int t) {
+    s2_cells(C.nx, C.rows, C.lf, t, [&](int R, int I) {
+        const int J = C.j0 + R, q = R * C.nx + I;
         const int ex = F.cfx == 1 ? 1 : (I == C.nx - 1 ? F.nx - 2 * I : 2);
         const int ey = F.cfy == 1 ? 1 : (J == C.ny - 1 ? F.ny - 2 * J : 2);
         const int i0 = F.cfx * I, j0 = F.cfy * J, base = (j0 - F.j0) * F.nx + i0;
@@ -215,58 +299,64 @@ PF_HD void s2_coarsen(const S2View<T>& F, const S2View<T>& C, int t, int nt) {
         };
         const float rx = dist(i0, F.nx, F.qx) / (float(F.cfx) * dist(I, C.nx, C.qx));
         const float ry = dist(j0, F.ny, F.qy) / (float(F.cfy) * dist(J, C.ny, C.qy));
-        // (the level's equations carry the factor h_0^2 of level 0: a quarter of
-        // MGLevel's coefficient, which multiplies ih2 of its own level)
-        C.w0[q] = C.nx == 1 ? T(0) : s0 * T(rx / float(vol));
-        C.w1[q] = C.ny == 1 ? T(0) : s1 * T(ry / float(vol));
-    }
+        // (the level's equations are those of MGLevel times h_0^2 and the cell's
+        // nominal volume over level 0's, so f is a plain sum of residuals)
+        C.w0[q] = C.nx == 1 ? T(0) : s0 * T(rx);
+        C.w1[q] = C.ny == 1 ? T(0) : s1 * T(ry);
+    });
 }
 
 PF_HD int s2_seams(int seams, int i, int j, int nx, int ny) {
     return ((seams & 1) && i == nx - 1) + ((seams & 2) && j == ny - 1);
 }
 
-// One class of a Gauss-Seidel sweep. zero: first class of a sweep that starts
-// from zero (on levels with odd or one-cell axes every other cell is set to
-// zero; on the others no cell is read before its class is written).
+// The first class of a sweep from zero, done where the right-hand side f of a
+// cell is formed: x = f / diagonal on the cells of class 0; on levels with odd
+// or one-cell axes zero on every other cell (on the others no cell is read
+// before its class is written).
 template <typename T>
-PF_HD void s2_gs(const S2View<T>& L, int cls, bool zero, int t, int nt) {
-    const int nx = L.nx, nhx = (nx + 1) >> 1, n = L.rows * nhx;
-    const int color = cls & 1, want = cls >> 1;
-    for (int q = t; q < n; q += nt) {
-        const int r = s2_div(q, L.inv_nhx);
-        const int m = q - r * nhx, j = L.j0 + r;
-        const int par = (j + color) & 1;
-        const int i = 2 * m + par, idx = r * nx + i;
-        if (!L.seams) {
-            L.x[idx] = (zero ? L.f[idx] : L.f[idx] + s2_off(L, r, i, idx)) * L.di[idx];
-            continue;
-        }
-        if (i < nx) {
-            if (s2_seams(L.seams, i, j, nx, L.ny) == want)
-                L.x[idx] = (zero ? L.f[idx] : L.f[idx] + s2_off(L, r, i, idx)) * L.di[idx];
-            else if (zero)
-                L.x[idx] = T(0);
-        }
-        const int o = 2 * m + 1 - par;
-        if (zero && o < nx) L.x[r * nx + o] = T(0);
+PF_HD void s2_start(const S2View<T>& L, int i, int j, int idx, T f) {
+    const bool c0 = ((i + j) & 1) == 0;
+    if (!L.seams) {
+        if (c0) L.x[idx] = f * L.di[idx];
+    } else {
+        L.x[idx] = c0 && s2_seams(L.seams, i, j, L.nx, L.ny) == 0 ? f * L.di[idx] : T(0);
     }
 }
 
-// f of the next level: residuals of the children over their nominal number.
-// After a sweep the residual of an even level's second colour is zero; with
-// one sweep from zero that of the first colour is the neighbours' part alone.
+// One class of a Gauss-Seidel sweep.
 template <typename T>
-PF_HD void s2_restrict(const S2View<T>& F, const S2View<T>& C, bool one_sweep, int t, int nt) {
-    const int n = C.rows * C.nx;
-    const T scale = T(1.0f / float(F.cfx * F.cfy));
-    for (int q = t; q < n; q += nt) {
-        const int R = s2_div(q, C.inv_nx);
-        const int I = q - R * C.nx, J = C.j0 + R;
+PF_HD void s2_gs(const S2View<T>& L, int cls, int t) {
+    const int nx = L.nx;
+    const int color = cls & 1, want = cls >> 1;
+    if (!L.seams) {
+        s2_map<T>(nx >> 1, L.rows, L.lh, t,
+                  [&](int r, int m) {
+                      const int i = 2 * m + ((L.j0 + r + color) & 1), idx = r * nx + i;
+                      return s2_off(L, r, i, idx, L.f[idx]) * L.di[idx];
+                  },
+                  [&](int r, int m, T v) { L.x[r * nx + 2 * m + ((L.j0 + r + color) & 1)] = v; });
+        return;
+    }
+    s2_cells((nx + 1) >> 1, L.rows, L.lh, t, [&](int r, int m) {
+        const int j = L.j0 + r, i = 2 * m + ((j + color) & 1), idx = r * nx + i;
+        if (i >= nx || s2_seams(L.seams, i, j, nx, L.ny) != want) return;
+        L.x[idx] = s2_off(L, r, i, idx, L.f[idx]) * L.di[idx];
+    });
+}
+
+// f of the next level (the sum of the children's residuals) and its sweep's
+// start. After a sweep the residual of an even level's second
+// colour is zero; with one sweep from zero that of the first colour is the
+// neighbours' part alone.
+template <typename T>
+PF_HD void s2_restrict(const S2View<T>& F, const S2View<T>& C, bool one_sweep, int t) {
+    auto value = [&](int R, int I) {
+        const int J = C.j0 + R;
         T s;
         if (!F.seams && F.cfx == 2 && F.cfy == 2) {
             const int r = 2 * J - F.j0, i = 2 * I, a = r * F.nx + i, b = a + F.nx + 1;
-            s = s2_off(F, r, i, a) + s2_off(F, r + 1, i + 1, b);
+            s = s2_off(F, r + 1, i + 1, b, s2_off(F, r, i, a, T(0)));
             if (!one_sweep)
                 s += (F.f[a] - s2_diag(F, r, i, a) * F.x[a]) +
                      (F.f[b] - s2_diag(F, r + 1, i + 1, b) * F.x[b]);
@@ -277,11 +367,16 @@ PF_HD void s2_restrict(const S2View<T>& F, const S2View<T>& C, bool one_sweep, i
             for (int b = 0; b < ey; ++b)
                 for (int e = 0; e < ex; ++e) {
                     const int i = F.cfx * I + e, r = F.cfy * J + b - F.j0, a = r * F.nx + i;
-                    s += F.f[a] - (s2_diag(F, r, i, a) * F.x[a] - s2_off(F, r, i, a));
+                    s += s2_off(F, r, i, a, F.f[a]) - s2_diag(F, r, i, a) * F.x[a];
                 }
         }
-        C.f[q] = s * scale;
-    }
+        return s;
+    };
+    s2_map<T>(C.nx, C.rows, C.lf, t, value, [&](int R, int I, T s) {
+        const int q = R * C.nx + I;
+        C.f[q] = s;
+        s2_start(C, I, C.j0 + R, q, s);
+    });
 }
 
 // Coarse neighbour (as an offset -1, 0, +1 from the parent I0) and its weight
@@ -295,12 +390,12 @@ PF_HD void s2_interp(int i, int nf, int nc, int cf, float qf, float qc, int& I0,
         return;
     }
     I0 = i >> 1;
-    if (I0 > nc - 1) I0 = nc - 1;
     if (qc == 1.f) {
         o = (i & 1) ? 1 : -1;
         w = T(0.25);
         return;
     }
+    if (I0 > nc - 1) I0 = nc - 1;
     const float wp = 2.f * (I0 == nc - 1 ? qc : 1.f);
     const float d = float(i - 2 * I0) + 0.5f * (i == nf - 1 ? qf : 1.f) - 0.5f * wp;
     o = d >= 0.f ? 1 : -1;
@@ -308,31 +403,216 @@ PF_HD void s2_interp(int i, int nf, int nc, int cf, float qf, float qc, int& I0,
     const bool l1 = (I1 < 0 ? nc - 1 : (I1 == nc ? 0 : I1)) == nc - 1;
     w = T((d < 0.f ? -d : d) / (0.5f * wp + (l1 ? qc : 1.f)));
 }
+template <typename T>
+PF_HD const T* s2_coarse_row(const S2View<T>& C, int R) {
+    return R < 0 ? C.xm : (R >= C.rows ? C.xp : C.x + R * C.nx);
+}
 
 // x += interpolation of the next level's x. On even levels only the first
 // colour: the post-sweep starts by overwriting the second.
 template <typename T>
-PF_HD void s2_prolong(const S2View<T>& F, const S2View<T>& C, int t, int nt) {
-    const bool half = !F.seams;
-    const int nx = F.nx, nh = half ? nx >> 1 : nx, n = F.rows * nh;
-    const float inv = half ? F.inv_nhx : F.inv_nx;
-    auto row = [&](int R) { return R < 0 ? C.xm : (R >= C.rows ? C.xp : C.x + R * C.nx); };
-    for (int q = t; q < n; q += nt) {
-        const int r = s2_div(q, inv), m = q - r * nh, j = F.j0 + r;
-        const int i = half ? 2 * m + (j & 1) : m;
+PF_HD void s2_prolong(const S2View<T>& F, const S2View<T>& C, int t) {
+    const int nx = F.nx;
+    const bool uniform = F.cfx == 2 && F.cfy == 2 && C.qx == 1.f && C.qy == 1.f;
+    auto value = [&](int r, int i) {
+        const int j = F.j0 + r;
         int I0, J0, oi, oj;
         T wi, wj;
         s2_interp<T>(i, nx, C.nx, F.cfx, F.qx, C.qx, I0, oi, wi);
         s2_interp<T>(j, F.ny, C.ny, F.cfy, F.qy, C.qy, J0, oj, wj);
         int I1 = I0 + oi;
         I1 = I1 < 0 ? C.nx - 1 : (I1 >= C.nx ? 0 : I1);
-        const int R0 = J0 - C.j0;
-        const T *c0 = row(R0), *c1 = row(R0 + oj);
+        const T *c0 = s2_coarse_row(C, J0 - C.j0), *c1 = s2_coarse_row(C, J0 - C.j0 + oj);
+        if (uniform) {
+            T v = F.x[r * nx + i] + T(0.5625) * c0[I0];
+            v += T(0.1875) * (c0[I1] + c1[I0]);
+            return v + T(0.0625) * c1[I1];
+        }
         const T a = c0[I0] + wi * (c0[I1] - c0[I0]);
         const T b = c1[I0] + wi * (c1[I1] - c1[I0]);
-        F.x[r * nx + i] += a + wj * (b - a);
+        return F.x[r * nx + i] + (a + wj * (b - a));
+    };
+    auto col = [&](int r, int m) { return 2 * m + ((F.j0 + r) & 1); };
+    if (!F.seams)
+        s2_map<T>(nx >> 1, F.rows, F.lh, t, [&](int r, int m) { return value(r, col(r, m)); },
+                  [&](int r, int m, T v) { F.x[r * nx + col(r, m)] = v; });
+    else
+        s2_map<T>(nx, F.rows, F.lf, t, value, [&](int r, int i, T v) { F.x[r * nx + i] = v; });
+}
+
+// The interpolation and the second colour of an even level's first post-sweep
+// in one phase: the first colour's interpolated values are formed by the cells
+// that read them (they are overwritten by the next class).
+template <typename T>
+PF_HD void s2_prolong_gs(const S2View<T>& F, const S2View<T>& C, int t) {
+    const int nx = F.nx;
+    s2_map<T>(nx >> 1, F.rows, F.lh, t, [&](int r, int m) {
+        const int j = F.j0 + r, par = (j + 1) & 1, i = 2 * m + par, idx = r * nx + i;
+        // parents' rows of fine row j (c0, its other neighbour c1); rows j - 1 and
+        // j + 1 share the parent of j or have it as their other neighbour
+        const int R = (j >> 1) - C.j0, I = m;
+        const int oj = (j & 1) ? 1 : -1;
+        const T *c0 = s2_coarse_row(C, R), *c1 = s2_coarse_row(C, R + oj);
+        const int Im = I == 0 ? C.nx - 1 : I - 1, Ip = I == C.nx - 1 ? 0 : I + 1;
+        // column interpolations of rows c0 and c1 at fine columns i - 1, i, i + 1
+        T a0[3], a1[3];
+        const T qt = T(0.25);
+        if (par) {   // i odd: i - 1 and i in parent I, i + 1 in parent Ip
+            const T x0 = c0[Im], x1 = c0[I], x2 = c0[Ip], y0 = c1[Im], y1 = c1[I], y2 = c1[Ip];
+            a0[0] = x1 + qt * (x0 - x1);
+            a0[1] = x1 + qt * (x2 - x1);
+            a0[2] = x2 + qt * (x1 - x2);
+            a1[0] = y1 + qt * (y0 - y1);
+            a1[1] = y1 + qt * (y2 - y1);
+            a1[2] = y2 + qt * (y1 - y2);
+        } else {     // i even: i - 1 in parent Im, i and i + 1 in parent I
+            const T x0 = c0[Im], x1 = c0[I], x2 = c0[Ip], y0 = c1[Im], y1 = c1[I], y2 = c1[Ip];
+            a0[0] = x0 + qt * (x1 - x0);
+            a0[1] = x1 + qt * (x0 - x1);
+            a0[2] = x1 + qt * (x2 - x1);
+            a1[0] = y0 + qt * (y1 - y0);
+            a1[1] = y1 + qt * (y0 - y1);
+            a1[2] = y1 + qt * (y2 - y1);
+        }
+        const T pl = a0[0] + qt * (a1[0] - a0[0]), pr = a0[2] + qt * (a1[2] - a0[2]);
+        // the sibling row (same parent) leans on the other side's coarse row; the
+        // row across the parent's edge has parent c1 and leans on c0
+        const T *c2 = s2_coarse_row(C, R - oj);
+        const int In = par ? Ip : Im;
+        const T b2 = c2[I] + qt * (c2[In] - c2[I]);
+        const T sib = a0[1] + qt * (b2 - a0[1]);
+        const T far = a1[1] + qt * (a0[1] - a1[1]);
+        const T pu = oj < 0 ? far : sib, pd = oj < 0 ? sib : far;
+        const S2Nb<T> n = s2_nb(F, r, i, idx);
+        const T wl = F.w0[idx], wr = F.w0[n.ir], wu = F.w1[idx], wd = *n.wd;
+        const T xl = F.x[n.il], xr = F.x[n.ir], xu = *n.xu, xd = *n.xd;
+        return (F.f[idx] + ((wl * (xl + pl) + wr * (xr + pr)) +
+                            (wu * (xu + pu) + wd * (xd + pd)))) * F.di[idx];
+    }, [&](int r, int m, T v) { F.x[r * nx + 2 * m + ((F.j0 + r + 1) & 1)] = v; });
+}
+
+// ---- dense level ----
+// M = pseudo-inverse of the level's A: the inverse of A + (sigma / n) 1 1^T
+// (symmetric positive definite) by Gauss-Jordan elimination without pivoting
+// (build, fill, n steps of elimination), with the means of its rows
+// and columns, weighted by A's diagonal, removed (means, then project). x is
+// defined up to a constant; this choice keeps it small where the coefficients
+// are large. A plain zero mean puts the light phase at the offset that the
+// heavy drop's large x asks for, and the rounding of A x there costs float32
+// solves at density ratio 1000 their convergence. A barrier follows each of
+// these functions.
+template <typename T>
+PF_HD void s2_dense_build(const S2View<T>& L, T* M, int t) {
+    const int n = L.nx * L.ny, ld = s2_pad(n);
+    T sig = T(0);
+    for (int k = 0; k < L.nx; ++k) sig += s2_diag(L, 0, k, k);
+    sig /= T(L.nx * n);
+    for (int q = t; q < n * ld; q += kS2Threads) M[q] = q % ld < n ? sig : T(0);
+}
+template <typename T>
+PF_HD void s2_dense_fill(const S2View<T>& L, T* M, int t) {
+    const int n = L.nx * L.ny, ld = s2_pad(n);
+    for (int a = t; a < n; a += kS2Threads) {
+        const int j = a / L.nx, i = a - j * L.nx;
+        T* row = M + a * ld;
+        const int il = j * L.nx + (i == 0 ? L.nx - 1 : i - 1), ir = j * L.nx + (i + 1 == L.nx ? 0 : i + 1);
+        const int iu = (j == 0 ? L.ny - 1 : j - 1) * L.nx + i, id = (j + 1 == L.ny ? 0 : j + 1) * L.nx + i;
+        const T w[4] = {L.w0[a], L.w0[ir], L.w1[a], L.w1[id]};
+        const int c[4] = {il, ir, iu, id};
+        for (int k = 0; k < 4; ++k) {
+            row[a] += w[k];
+            row[c[k]] -= w[k];
+        }
     }
 }
+// Elimination: a thread keeps its eight elements (column t % 64, rows t / 64 +
+// 8 i) in registers; publish copies column k, row k and the pivot's reciprocal
+// of the current matrix into one of two buffers, step reads them. One barrier
+// a step.
+constexpr int kS2Col = 64, kS2ColRow = 129;   // offsets of the row; elements of a buffer
+template <typename T>
+PF_HD void s2_gj_publish(const T (&m)[8], int n, int k, T* buf, int t) {
+    const int c = t & 63, r0 = t >> 6;
+    if (c >= n || k >= n) return;
+    if (c == k) {
+        for (int i = 0; i < 8; ++i)
+            if (r0 + 8 * i < n) buf[r0 + 8 * i] = m[i];
+    }
+    if (r0 == (k & 7)) {
+        T v = m[0];
+        for (int i = 1; i < 8; ++i) v = i == (k >> 3) ? m[i] : v;
+        buf[kS2Col + c] = v;
+        if (c == k) buf[128] = T(1) / v;
+    }
+}
+template <typename T>
+PF_HD void s2_gj_step(T (&m)[8], int n, int k, const T* buf, int t) {
+    const int c = t & 63, r0 = t >> 6;
+    if (c >= n) return;
+    const T rk = (c == k ? T(1) : buf[kS2Col + c]) * buf[128];
+    for (int i = 0; i < 8; ++i) {
+        const int r = r0 + 8 * i;
+        if (r >= n) continue;
+        m[i] = r == k ? rk : (c == k ? T(0) : m[i]) - buf[r] * rk;
+    }
+}
+template <typename T>
+PF_HD void s2_gj_move(T (&m)[8], T* M, int n, bool store, int t) {
+    const int c = t & 63, ld = s2_pad(n);
+    for (int i = 0; i < 8; ++i) {
+        const int r = (t >> 6) + 8 * i;
+        if (c < n && r < n) {
+            if (store) M[r * ld + c] = m[i];
+            else m[i] = M[r * ld + c];
+        }
+    }
+}
+// (k = 0: the weights; 1: row and column means; 2: their mean)
+template <typename T>
+PF_HD void s2_dense_means(const S2View<T>& L, const T* M, int n, int k, T* colrow, int t) {
+    const int ld = s2_pad(n);
+    T* d = colrow + kS2ColRow;   // (the second buffer)
+    if (k == 0) {
+        if (t < n) {
+            const int r = t / L.nx, i = t - r * L.nx;
+            d[t] = s2_diag(L, r, i, t);
+        }
+        return;
+    }
+    T s = T(0), w = T(0);
+    if (k == 1 && (t < n || (t >= 64 && t < 64 + n))) {
+        for (int c = 0; c < n; ++c) {
+            s += d[c] * (t < 64 ? M[t * ld + c] : M[c * ld + t - 64]);
+            w += d[c];
+        }
+        colrow[t] = s / w;
+    } else if (k == 2 && t == 128) {
+        for (int c = 0; c < n; ++c) {
+            s += d[c] * colrow[c];
+            w += d[c];
+        }
+        colrow[t] = s / w;
+    }
+}
+template <typename T>
+PF_HD void s2_dense_project(T* M, int n, const T* colrow, int t) {
+    const int ld = s2_pad(n), c = t & 63;
+    if (c < n)
+        for (int r = t >> 6; r < n; r += kS2Threads >> 6)
+            M[r * ld + c] -= (colrow[r] + colrow[64 + c]) - colrow[128];
+}
+// x = M f of the part of thread t: row t / 8, every eighth column from t % 8
+template <typename T>
+PF_HD T s2_dense_part(const T* M, const T* f, int n, int t) {
+    const int r = t >> 3;
+    T s = T(0);
+    if (r < n) {
+        const T* row = M + r * s2_pad(n);
+        for (int c = t & 7; c < n; c += 8) s += row[c] * f[c];
+    }
+    return s;
+}
+constexpr int kS2DenseMax = kS2Threads / 8;   // cells of a dense level
 
 // Sums whose rounding is carried along: float64 sums of the float64 path,
 // (hi, lo) float pairs of the mixed one (a float64 accumulation without GB300's
@@ -366,74 +646,81 @@ template <> struct S2AccOf<float> { using type = S2AccF; };
 // The last class (0) of the last post-sweep of level 0 with the CG products
 // rz = f.x and, unless first, zq = x.q over every cell of the strip.
 template <typename T, typename A>
-PF_HD void s2_gs_dots(const S2View<T>& L, const T* qv, bool first, A& rz, A& zq, int t, int nt) {
-    const int nx = L.nx, nhx = (nx + 1) >> 1, n = L.rows * nhx;
-    for (int q = t; q < n; q += nt) {
-        const int r = s2_div(q, L.inv_nhx);
-        const int m = q - r * nhx, j = L.j0 + r;
-        const int par = j & 1;
-        const int i = 2 * m + par, o = 2 * m + 1 - par;
+PF_HD void s2_gs_dots(const S2View<T>& L, const T* qv, bool first, A& rz, A& zq, int t) {
+    const int nx = L.nx;
+    s2_map<T>((nx + 1) >> 1, L.rows, L.lh, t, [&](int r, int m) {
+        const int j = L.j0 + r, par = j & 1, i = 2 * m + par, o = 2 * m + 1 - par;
+        T x = T(0);
         if (i < nx) {
             const int idx = r * nx + i;
             const T f = L.f[idx];
-            T x;
-            if (!L.seams || s2_seams(L.seams, i, j, nx, L.ny) == 0) {
-                x = (f + s2_off(L, r, i, idx)) * L.di[idx];
-                L.x[idx] = x;
-            } else {
-                x = L.x[idx];
-            }
+            x = !L.seams || s2_seams(L.seams, i, j, nx, L.ny) == 0
+                    ? s2_off(L, r, i, idx, f) * L.di[idx] : L.x[idx];
             rz.add_prod(f, x);
             if (!first) zq.add_prod(x, qv[idx]);
         }
         if (o < nx) {
             const int idx = r * nx + o;
-            const T x = L.x[idx];
-            rz.add_prod(L.f[idx], x);
-            if (!first) zq.add_prod(x, qv[idx]);
+            const T y = L.x[idx];
+            rz.add_prod(L.f[idx], y);
+            if (!first) zq.add_prod(y, qv[idx]);
         }
-    }
+        return x;
+    }, [&](int r, int m, T x) {
+        const int i = 2 * m + ((L.j0 + r) & 1);
+        if (i < nx) L.x[r * nx + i] = x;
+    });
 }
 
 // p = z + beta p (first: p = z)
 template <typename T>
-PF_HD void s2_direction(const S2View<T>& L, T* p, T beta, bool first, int t, int nt) {
-    const int n = L.rows * L.nx;
-    for (int q = t; q < n; q += nt) p[q] = first ? L.x[q] : L.x[q] + beta * p[q];
+PF_HD void s2_direction(const S2View<T>& L, T* p, T beta, bool first, int t) {
+    s2_map<T>(L.nx, L.rows, L.lf, t, [&](int r, int i) {
+        const int k = r * L.nx + i;
+        return first ? L.x[k] : L.x[k] + beta * p[k];
+    }, [&](int r, int i, T v) { p[r * L.nx + i] = v; });
 }
 
 // q = A p and p.q; pm, pp: the rows of p around the strip
 template <typename T, typename A>
-PF_HD void s2_apply(const S2View<T>& L, const T* p, const T* pm, const T* pp, T* qv, A& pq, int t,
-                    int nt) {
-    const int nx = L.nx, n = L.rows * nx;
-    for (int q = t; q < n; q += nt) {
-        const int r = s2_div(q, L.inv_nx), i = q - r * nx;
+PF_HD void s2_apply(const S2View<T>& L, const T* p, const T* pm, const T* pp, T* qv, A& pq, int t) {
+    const int nx = L.nx;
+    s2_map<T>(nx, L.rows, L.lf, t, [&](int r, int i) {
+        const int q = r * nx + i;
         const int il = i == 0 ? q + nx - 1 : q - 1;
         const int ir = i == nx - 1 ? q - i : q + 1;
         const bool last = r == L.rows - 1;
-        const T pc = p[q];
-        T ax = L.w0[q] * (pc - p[il]);
-        ax += L.w0[ir] * (pc - p[ir]);
-        ax += L.w1[q] * (pc - (r == 0 ? pm[i] : p[q - nx]));
-        ax += (last ? L.w1p[i] : L.w1[q + nx]) * (pc - (last ? pp[i] : p[q + nx]));
-        qv[q] = ax;
+        const T* pu = r == 0 ? pm + i : p + (q - nx);
+        const T* pd = last ? pp + i : p + (q + nx);
+        const T* wd = last ? L.w1p + i : L.w1 + (q + nx);
+        const T pc = p[q], w0 = L.w0[q], wr = L.w0[ir], w1 = L.w1[q], w3 = *wd;
+        const T xl = p[il], xr = p[ir], xu = *pu, xd = *pd;
+        T ax = w0 * (pc - xl);
+        ax += wr * (pc - xr);
+        ax += w1 * (pc - xu);
+        ax += w3 * (pc - xd);
         pq.add_prod(pc, ax);
-    }
+        return ax;
+    }, [&](int r, int i, T v) { qv[r * nx + i] = v; });
 }
 
-// e += alpha p, r -= alpha q (r: the level's f), per-thread sum of r^2
+// e += alpha p, r -= alpha q (r: the level's f), the next sweep's start;
+// per-thread sum of r^2
 template <typename T>
-PF_HD T s2_update(const S2View<T>& L, const T* p, const T* qv, T* e, T alpha, bool first, int t,
-                  int nt) {
-    const int n = L.rows * L.nx;
+PF_HD T s2_update(const S2View<T>& L, const T* p, const T* qv, T* e, T alpha, bool first, int t) {
+    const int nx = L.nx;
     T rr = T(0);
-    for (int q = t; q < n; q += nt) {
-        e[q] = first ? alpha * p[q] : e[q] + alpha * p[q];
-        const T rv = L.f[q] - alpha * qv[q];
-        L.f[q] = rv;
-        rr += rv * rv;
-    }
+    struct ER { T e, r; };
+    s2_map<ER>(nx, L.rows, L.lf, t, [&](int r, int i) {
+        const int k = r * nx + i;
+        return ER{first ? alpha * p[k] : e[k] + alpha * p[k], L.f[k] - alpha * qv[k]};
+    }, [&](int r, int i, ER v) {
+        const int k = r * nx + i;
+        e[k] = v.e;
+        L.f[k] = v.r;
+        s2_start(L, i, L.j0 + r, k, v.r);
+        rr += v.r * v.r;
+    });
     return rr;
 }
 

@@ -63,3 +63,34 @@ def test_solve_on_any_size(pf, n, precision):
     assert np.linalg.norm(x - want) <= (1.01 * rtol + 2.0 ** -40) * np.linalg.norm(f) / lam
     # a V-cycle that halves the error per iteration or better
     assert iters <= np.log2(1.0 / rtol) + 4
+
+
+@pytest.mark.parametrize("n,ratio", [((64, 64), 1000.0), ((256, 256), 1000.0), ((320, 320), 10.0),
+                                     ((512, 40), 10.0), ((384, 512), 10.0), ((512, 512), 10.0),
+                                     ((650, 650), 10.0), ((700, 700), 10.0)])
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("sweeps", [1, 2])
+def test_2d_solve_residual(pf, n, ratio, precision, sweeps):
+    """Strips of unequal rows, arrays that overflow into the workspace, the
+    largest grids of the one-launch solve and the multi-kernel solve beyond it:
+    the residual of the returned x, formed here, meets the tolerance."""
+    rtol = 1e-10
+    p = I.small_case(dim=2, n=n[0], precision=precision, poisson_rtol=rtol, rho_in=10.0,
+                     rho_out=10.0 / ratio, mg_pre=sweeps, mg_post=sweeps)
+    p["n"] = n + (1,)
+    p = I.finalize(p)
+    po = O.params_from(p)
+    g = O.Grid(2, n, p["L"])
+    phi = O.initial_phi(po).astype(np.float32).astype(np.float64)
+    rhs = I.noise(g.shape, 6) - 0.5
+    rhs -= rhs.mean()
+    sim = pf.Simulation(p, phi0=phi)
+    x, iters, rel, status = sim.poisson_solve(rhs)
+    sim.close()
+    beta = O.face_beta(phi, g, po) if precision == "fp64" else beta32(phi, g, p)
+    r = rhs - O.apply_poisson(beta, x, g)
+    # rounding of x (2^-47 for a double-float, 2^-52 for float64) through the operator
+    eps = 2.0 ** -47 if precision == "mixed" else 2.0 ** -52
+    floor = 8.0 * eps * max(b.max() for b in beta) / g.h ** 2 * np.linalg.norm(x)
+    assert status == 0 and iters <= 40
+    assert np.linalg.norm(r) <= 1.01 * rtol * np.linalg.norm(rhs) + floor
