@@ -10,6 +10,7 @@
 
 #include "../../include/pf.h"
 #include "pf_internal.h"
+#include "pf_coarse3d.cuh"
 #include "pf_solve2d.cuh"
 
 using namespace pf;
@@ -362,11 +363,38 @@ struct ImplT final : Impl {
         // 1/4 (three cells in 3D, uniform density) or more a sweep
         const int sweeps = nmax <= 2 ? 4 : (nmax == 3 ? 5 : 4 * nmax * nmax);
         H.coarse_sweeps = sweeps > 2000 ? 2000 : sweeps;
+        // 3D: the coarse levels in one cluster launch, by default from the finest
+        // coarse level that fits (a caller's mg_coarse_cells names the level)
+        H.c3 = nullptr;
+        if (DIM == 3 && !even_only) {
+            int l0 = H.first_coarse;
+            bool ok = false;
+            if (prm.mg_coarse_cells == 0)
+                for (int l = 1; l < l0 && !ok; ++l)
+                    if (H.lev[l].g.ncell <= 40000 && coarse3d_plan<T>(H, l, c3)) {
+                        ok = true;
+                        l0 = l;
+                    }
+            if (!ok) ok = coarse3d_plan<T>(H, l0, c3);
+            if (ok) {
+                H.first_coarse = l0;
+                H.c3 = &c3;
+            }
+        }
+    }
+    void carve_coarse3d(Carver& cv) {
+        H.c3_di = H.c3_minv = nullptr;
+        if (!H.c3) return;
+        size_t nd = 0, nm = 0;
+        coarse3d_sizes<T>(c3, &nd, &nm);
+        H.c3_di = cv.take<T>(nd);
+        H.c3_minv = cv.take<T>(nm);
     }
 
     bool owns_host = false;
     cudaEvent_t sleep_ev = nullptr;   // blocking-sync event (batched execution)
 
+    C3Plan c3;                 // cluster launch of the 3D coarse levels (H.c3 points here)
     S2Plan s2;                 // one-launch solve of 2D grids that fit (s2_state 1; 0 not decided,
     int s2_state = 0;          // 2 the multi-kernel solve)
 
@@ -473,6 +501,7 @@ struct ImplT final : Impl {
             for (int l = 1; l < H.first_coarse && l <= kDensityLevels; ++l)
                 H.rhoc[l] = sweep3d_ok(H.lev[l].g) && sweep3d_ok(H.lev[l - 1].g)
                                 ? cv.take<float>(H.lev[l].g.ncell) : nullptr;
+        carve_coarse3d(cv);
         rb.part = cv.take<double>(kRedPart);
         rb.counter = cv.take<unsigned int>(4);
         sc = cv.take<CGScalars>(1);
@@ -506,6 +535,7 @@ struct ImplT final : Impl {
             H.lev[l].f = cv.take<T>(m);
             for (int d = 0; d < 3; ++d) H.lev[l].beta[d] = d < DIM ? cv.take<T>(m) : nullptr;
         }
+        carve_coarse3d(cv);
         rb.part = cv.take<double>(kRedPart);
         rb.counter = cv.take<unsigned int>(4);
         sc = cv.take<CGScalars>(1);
@@ -885,6 +915,7 @@ struct ImplT final : Impl {
         sweep_tma_prepare();
         stage_fused_prepare();
         coarse_prepare();
+        coarse3d_prepare();
         if (DIM == 2) use_solve2d();
         // the legacy default stream cannot be captured: record on a private
         // stream (recording runs nothing); the graph replays on the context's
@@ -1555,8 +1586,8 @@ pf_status run_static_solve(const pf_params& prm, cudaStream_t st, void* scratch,
     Carver size_cv{nullptr};
     im.carve_solver_only(size_cv);
     if (size_cv.off > (size_t)PF_STATIC_SCRATCH_BYTES) {
-        // odd sizes coarsened add levels: a grid that fits without them is solved
-        // without them
+        // odd sizes coarsened add levels, and the cluster launch of the coarse levels
+        // its scratch: a grid that fits without them is solved without them
         im.build_levels(true);
         size_cv.off = 0;
         im.carve_solver_only(size_cv);

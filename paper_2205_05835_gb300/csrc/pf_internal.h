@@ -154,8 +154,14 @@ struct MGHier {
                                    // formed (3D mixed path; nullptr elsewhere)
     const SweepTMA* tma = nullptr; // level 0 sweeps staged by the TMA (nullptr: cp.async)
     const SweepTMA* tmac[kMaxLevels] = {};   // the same for the levels l >= 1 with densities
+    // 3D: the coarse part of a V-cycle in one cluster launch (pf_coarse3d.cu): the
+    // plan (host object; nullptr: the single-CTA kernel), the levels' inverse
+    // diagonals and the dense level's inverse
+    const struct C3Plan* c3 = nullptr;
+    T* c3_di = nullptr;
+    T* c3_minv = nullptr;
     int nlev;
-    int first_coarse;   // levels >= first_coarse are handled by one single-CTA kernel
+    int first_coarse;   // levels >= first_coarse are handled by one kernel
     int pre, post;
     int coarse_sweeps;
     MGLevel<T> lev[kMaxLevels];
@@ -355,6 +361,19 @@ void launch_in_dir(const Dims& g, const Phys& ph, const SolveIO<T, DIM>& io, int
 template <typename T, int DIM>
 void launch_in_update(const Dims& g, const SolveIO<T, DIM>& io, int cur, int first, RedBuf rb,
                       CGScalars* sc, cudaStream_t s);
+// The coarse levels of a 3D V-cycle in one launch of a thread-block cluster
+// (pf_coarse3d.cu). Plan for the levels >= l0 (false: they do not fit), the
+// elements of c3_di / c3_minv, the once-per-solve setup and the launch.
+struct C3Plan;
+void coarse3d_prepare();
+template <typename T>
+bool coarse3d_plan(const MGHier<T>& H, int l0, C3Plan& P);
+template <typename T>
+void coarse3d_sizes(const C3Plan& P, size_t* di, size_t* minv);
+template <typename T>
+void launch_coarse3d_setup(const C3Plan& P, const MGHier<T>& H, cudaStream_t s);
+template <typename T>
+void launch_coarse3d(const C3Plan& P, const MGHier<T>& H, const CGScalars* sc, cudaStream_t s);
 // The whole 2D solve in one launch of a thread-block cluster (pf_solve2d.cu).
 // solve2d_plan: false when the grid does not fit (use the kernels above).
 // b0, b1: the face coefficients of level 0, written (null: none are kept).

@@ -687,6 +687,12 @@ void coarse_smem_attribute() {
     });
 }
 
+// the cluster kernel reads the face coefficients of every level it holds
+template <typename T>
+static bool use_coarse3d(const MGHier<T>& H) {
+    return H.c3 != nullptr && H.c3_di != nullptr && H.lev[H.first_coarse].beta[0] != nullptr;
+}
+
 template <typename T, int DIM>
 void launch_mg_setup(const Dims&, const Phys& ph, const T* phi, MGHier<T>& H, cudaStream_t s) {
     for (int l = 0; l + 1 < H.nlev; ++l) {
@@ -702,6 +708,7 @@ void launch_mg_setup(const Dims&, const Phys& ph, const T* phi, MGHier<T>& H, cu
         k_coarsen_beta<T, DIM><<<row_grid(H.lev[l + 1].g, kThreads, 1 << 30), kThreads, 0, s>>>(
             H.lev[l], H.lev[l + 1], phi, ph);
     }
+    if (DIM == 3 && use_coarse3d(H)) launch_coarse3d_setup<T>(*H.c3, H, s);
 }
 
 template <typename T, int DIM>
@@ -794,7 +801,9 @@ T* launch_vcycle(const Phys& ph, const T* phi, MGHier<T>& H, const CGScalars* sc
     }
     pr->begin(KC_COARSE);
     const size_t cbytes = coarse_smem_bytes<T, DIM>(H);
-    if (cbytes > 0) {
+    if (DIM == 3 && use_coarse3d(H)) {
+        launch_coarse3d<T>(*H.c3, H, sc, s);
+    } else if (cbytes > 0) {
         coarse_smem_attribute<T, DIM>();
         k_coarse_vcycle_smem<T, DIM><<<1, kCoarseThreads, cbytes, s>>>(H, phi, ph, sc);
     } else {

@@ -13,6 +13,7 @@
 #include <mutex>
 #include <type_traits>
 
+#include "pf_cluster.cuh"
 #include "pf_device.cuh"
 #include "pf_solve2d.cuh"
 
@@ -35,27 +36,6 @@ struct S2Args {
     T *gdi, *gp, *gq, *ge;
     CGScalars* sc;
 };
-
-__device__ __forceinline__ int cluster_rank() {
-    int r;
-    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-// the address in CTA `rank` of the cluster of a shared-memory address of this CTA
-template <typename T>
-__device__ __forceinline__ T* cluster_map(T* p, int rank) {
-    T* q;
-    asm("mapa.u64 %0, %1, %2;" : "=l"(q) : "l"(p), "r"(rank));
-    return q;
-}
-__device__ __forceinline__ void cluster_sync(int C) {
-    if (C == 1) {
-        __syncthreads();
-    } else {
-        asm volatile("barrier.cluster.arrive.release.aligned;\n"
-                     "barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    }
-}
 
 // ---- totals over the cluster ----
 __device__ __forceinline__ S2AccF shfl_acc(S2AccF a, int o) {
@@ -391,8 +371,10 @@ __global__ void __launch_bounds__(kS2Threads, 1) k_solve2d(const __grid_constant
         }
         s2_gj_move(m, M, n, true, tid);
         __syncthreads();
-        for (int k = 0; k < 3; ++k) {
-            s2_dense_means(S[ld], M, n, k, colrow, tid);
+        s2_dense_weights(S[ld], colrow + kS2ColRow, tid);
+        __syncthreads();
+        for (int k = 1; k < 3; ++k) {
+            s2_dense_means(M, n, k, colrow, tid);
             __syncthreads();
         }
         s2_dense_project(M, n, colrow, tid);

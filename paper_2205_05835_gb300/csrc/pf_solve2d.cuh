@@ -567,18 +567,19 @@ PF_HD void s2_gj_move(T (&m)[8], T* M, int n, bool store, int t) {
         }
     }
 }
-// (k = 0: the weights; 1: row and column means; 2: their mean)
+// the weights, in the second buffer
 template <typename T>
-PF_HD void s2_dense_means(const S2View<T>& L, const T* M, int n, int k, T* colrow, int t) {
-    const int ld = s2_pad(n);
-    T* d = colrow + kS2ColRow;   // (the second buffer)
-    if (k == 0) {
-        if (t < n) {
-            const int r = t / L.nx, i = t - r * L.nx;
-            d[t] = s2_diag(L, r, i, t);
-        }
-        return;
+PF_HD void s2_dense_weights(const S2View<T>& L, T* d, int t) {
+    if (t < L.nx * L.ny) {
+        const int r = t / L.nx, i = t - r * L.nx;
+        d[t] = s2_diag(L, r, i, t);
     }
+}
+// (k = 1: row and column means; 2: their mean)
+template <typename T>
+PF_HD void s2_dense_means(const T* M, int n, int k, T* colrow, int t) {
+    const int ld = s2_pad(n);
+    const T* d = colrow + kS2ColRow;
     T s = T(0), w = T(0);
     if (k == 1 && (t < n || (t >= 64 && t < 64 + n))) {
         for (int c = 0; c < n; ++c) {
