@@ -126,6 +126,7 @@ struct MGLevel {
     T* f;          // right-hand side
     T* beta[3];    // face coefficients 1/rho_f (nullptr on level 0: computed from phi)
     T* x2;         // second correction buffer for out-of-place sweeps (nullptr: in place)
+    T* di;         // inverse diagonals (float64 levels of the multi-kernel V-cycle; nullptr: none)
     // Coarsening to the next level: factor cf[d] (2, or 1 where an axis has one
     // cell) and n[d] / cf[d] coarse cells, the last of which takes three
     // children where n[d] is odd. lastw[d]: width of the last cell
@@ -254,6 +255,28 @@ struct DiagOut {
     double nonfinite;
 };
 
+// Planes per CTA of a kernel that marches cols column tiles in z: the chunk with
+// the least modelled time, max(1, CTAs / slots) (zc + extra), slots the CTAs
+// resident at once and extra the planes' worth of halo and pipeline start that
+// a chunk pays. Many short chunks (8 CTAs per SM and more) pay it several
+// times over: at 128^3 a sweep from x_in takes 29 us with 14-plane chunks and
+// 48 us with 4-plane ones, the direction kernel 20 and 27 us; at 384^3 chunks
+// of 48 to 96 planes differ by 2 %.
+inline int march_zc(long long cols, int nz, long long slots, int extra, int zmax = 64) {
+    int best = 2;
+    double cost = 1e300;
+    for (int zc = 2; zc <= zmax && zc <= nz; ++zc) {
+        const long long b = cols * ((nz + zc - 1) / zc);
+        const double w = b > slots ? double(b) / double(slots) : 1.0;
+        const double c = w * double(zc + extra);
+        if (c <= cost) {
+            cost = c;
+            best = zc;
+        }
+    }
+    return best;
+}
+
 // Kernel classes timed by the optional profiler.
 enum KernelClass {
     KC_CELL = 0, KC_STAGE, KC_GAMMA, KC_DIV, KC_CORRECT, KC_COARSEN, KC_GS0, KC_GS,
@@ -378,6 +401,7 @@ void launch_coarse3d(const C3Plan& P, const MGHier<T>& H, const CGScalars* sc, c
 // solve2d_plan: false when the grid does not fit (use the kernels above).
 // b0, b1: the face coefficients of level 0, written (null: none are kept).
 struct S2Plan;
+constexpr int kSolve2dCells64 = 16 * 16500;   // float64 grids above do not take it
 void solve2d_prepare();
 template <typename T>
 bool solve2d_plan(const MGHier<T>& H, bool beta_global, S2Plan& P);

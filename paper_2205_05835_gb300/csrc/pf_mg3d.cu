@@ -392,8 +392,8 @@ void launch_sweep3d_t(const SweepArgs& a, dim3 grid, const CGScalars* sc, cudaSt
 
 }  // namespace
 
-// z chunk of the tiled kernels: enough CTAs to fill the GPU (about 8 per SM),
-// 2..32 planes each
+// bound on the CTAs of the tiled kernels: chunks of 2..32 planes, about 8 CTAs
+// per SM
 int tiled_zc(const Dims& g) {
     const int cols = ((g.nx + TX - 1) / TX) * ((g.ny + TY - 1) / TY);
     int zc = 32;
@@ -445,13 +445,9 @@ void launch_sweep3d(const MGLevel<float>& L, const float* phi, int rho_ready, co
         a.rb = RedBuf{nullptr, nullptr};
         a.scw = nullptr;
     }
-    // 64-plane chunks where that still gives 8 CTAs per SM (the z halo and
-    // the pipeline start are paid once per chunk), else the shared choice
-    int zc = tiled_zc(L.g);
-    {
-        const long long cols = (long long)((L.g.nx + TX - 1) / TX) * ((L.g.ny + TY - 1) / TY);
-        if (zc == 32 && cols * ((L.g.nz + 63) / 64) >= 8 * 152) zc = 64;
-    }
+    // the chunks of the TMA-staged sweep's default tiles (the same partial sums)
+    const long long cols = (long long)((L.g.nx + TX - 1) / TX) * ((L.g.ny + TY - 1) / TY);
+    const int zc = march_zc(cols, L.g.nz, 152 * (xin == nullptr ? 6 : 4), 6);
     a.zc = zc;
     dim3 grid((L.g.nx + TX - 1) / TX, (L.g.ny + TY - 1) / TY, (L.g.nz + zc - 1) / zc);
     if (dots && 2LL * grid.x * grid.y * grid.z > (long long)kRedPart) {
@@ -676,7 +672,9 @@ void launch_dir3d_reg(const Dims& g, const float* z, const float* p_old, float* 
     a.first = first;
     a.rb = rb;
     a.sc = sc;
-    const int zc = tiled_zc(g);
+    const long long cols = (long long)((g.nx + 31) / 32) * ((g.ny + 7) / 8);
+    int zc = march_zc(cols, g.nz, 4 * 152, 6);
+    if (cols * ((g.nz + zc - 1) / zc) > kRedPart) zc = tiled_zc(g);
     a.zc = zc;
     dim3 grid((g.nx + 31) / 32, (g.ny + 7) / 8, (g.nz + zc - 1) / zc);
     if (rho)
@@ -834,7 +832,9 @@ void launch_ir_residual3d(const Dims& g, const float* x, const float* b, const f
     a.first = first;
     a.rb = rb;
     a.sc = sc;
-    const int zc = tiled_zc(g);
+    const long long cols = (long long)((g.nx + 31) / 32) * ((g.ny + 7) / 8);
+    int zc = march_zc(cols, g.nz, 5 * 152, 6);
+    if (3 * cols * ((g.nz + zc - 1) / zc) > kRedPart) zc = tiled_zc(g);
     a.zc = zc;
     dim3 grid((g.nx + 31) / 32, (g.ny + 7) / 8, (g.nz + zc - 1) / zc);
     k_ir_residual3d<<<grid, 256, 0, s>>>(a);

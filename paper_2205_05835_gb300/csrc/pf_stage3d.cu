@@ -240,8 +240,12 @@ void launch_cell_pass_mu3d(const Dims& g, const Phys& ph, const float* phi, floa
     k_cell_pass_mu3d<<<zgrid(g, a.zc), ZT, 0, s>>>(a);
 }
 
+int divergence_zc(const Dims& g) {
+    const long long cols = (long long)((g.nx + ZX - 1) / ZX) * ((g.ny + ZY - 1) / ZY);
+    return march_zc(cols, g.nz, 6 * 152, 6);
+}
 bool divergence3d_ok(const Dims& g) {
-    const int zc = zchunk(g);
+    const int zc = divergence_zc(g);
     const dim3 gr = zgrid(g, zc);
     return g.nz > 1 && (long long)gr.x * gr.y * gr.z <= kRedPart;
 }
@@ -257,7 +261,7 @@ void launch_divergence3d(const Dims& g, const float* const* u, double inv_tau, d
     a.b = b;
     a.rb = rb;
     a.sc = sc;
-    a.zc = zchunk(g);
+    a.zc = divergence_zc(g);
     k_divergence3d<<<zgrid(g, a.zc), ZT, 0, s>>>(a);
 }
 

@@ -502,10 +502,9 @@ template <int TY, int CPT>
 void launch_tiles(const SweepTMA* t, const CUtensorMap* tx, TmaArgs& a, bool zero,
                   const SweepDots* dots, bool* ok, const CGScalars* sc, cudaStream_t s) {
     const Dims& g = t->g;
-    int zc = 32;
     const long long cols = (long long)((g.nx + TX - 1) / TX) * ((g.ny + TY - 1) / TY);
-    while (zc > 2 && cols * ((g.nz + zc - 1) / zc) < 8 * 152) zc >>= 1;
-    if (zc == 32 && cols * ((g.nz + 63) / 64) >= 8 * 152) zc = 64;
+    const int zc = march_zc(cols, g.nz, 152 * (zero ? tile_min_blocks<true, TY, CPT>()
+                                                    : tile_min_blocks<false, TY, CPT>()), 6);
     a.zc = zc;
     dim3 grid((g.nx + TX - 1) / TX, (g.ny + TY - 1) / TY, (g.nz + zc - 1) / zc);
     *ok = !(dots && 2LL * grid.x * grid.y * grid.z > (long long)kRedPart);
