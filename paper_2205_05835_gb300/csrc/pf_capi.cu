@@ -486,6 +486,11 @@ struct ImplT final : Impl {
             H.lev[l].f = cv.take<T>(m);
             for (int d = 0; d < 3; ++d) H.lev[l].beta[d] = d < DIM ? cv.take<T>(m) : nullptr;
         }
+        // inverse diagonals of the float64 levels outside the coarse kernel (2D:
+        // grids beyond the one-launch solve)
+        for (int l = 0; l < kMaxLevels; ++l) H.lev[l].di = nullptr;
+        if (sizeof(T) == sizeof(double) && (DIM == 3 || n > (size_t)kSolve2dCells64))
+            for (int l = 0; l < H.first_coarse; ++l) H.lev[l].di = cv.take<T>(H.lev[l].g.ncell);
         // second buffers for the one-pass out-of-place sweeps (3D float32 levels
         // below the single-CTA levels)
         if (DIM == 3 && sizeof(T) == sizeof(float))
@@ -513,6 +518,7 @@ struct ImplT final : Impl {
     // Layout of a pressure solve alone (phi plus the solver's vectors), used by
     // the allocation-free entry point; the stage fields stay unset.
     void carve_solver_only(Carver& cv) {
+        for (int l = 0; l < kMaxLevels; ++l) H.lev[l].di = nullptr;
         const size_t n = g.ncell;
         phiN = cv.take<T>(n);
         p = cv.take<double>(n);

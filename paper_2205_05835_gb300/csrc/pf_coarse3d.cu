@@ -1,6 +1,6 @@
 // The coarse part of a 3D V-cycle in one launch of a thread-block cluster: the
 // levels from about 32^3 cells down, each level's arrays in shared memory,
-// slabs of planes per CTA, the level of at most 64 (float64: 27) cells solved
+// slabs of planes per CTA, the level of at most 27 cells solved
 // by its inverse. It replaces, per V-cycle, four launches per level of a few
 // thousand cells (4 to 5 us each) and a single-CTA kernel whose ~70 dependent
 // phases took 41 us at 16^3 in float32 and 118 us at 12^3 in float64.
@@ -58,12 +58,12 @@ __global__ void __launch_bounds__(kS2Threads) k_c3_setup(const __grid_constant__
     T* M = reinterpret_cast<T*>(c3_raw);
     __shared__ C3View<T> v;
     __shared__ T colrow[2 * kS2ColRow];
-    __shared__ T w[3][64];
+    __shared__ T w[3][kS2DenseMax];
     const C3Lev& L = P.lev[P.ld];
     const int n = L.nx * L.ny * L.nz;
     const T kap = T(P.kappa[P.ld]);
-    if (tid < 3 * 64) {
-        const int d = tid >> 6, q = tid & 63;
+    if (tid < 3 * kS2DenseMax) {
+        const int d = tid / kS2DenseMax, q = tid % kS2DenseMax;
         if (q < n) w[d][q] = kap * a.beta[P.ld][d][q];
     }
     if (tid == 0) {
@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(kS2Threads) k_c3_setup(const __grid_constant__
     __syncthreads();
     c3_dense_fill(v, M, tid);
     __syncthreads();
-    T m[8];
+    T m[2];
     s2_gj_move(m, M, n, false, tid);
     s2_gj_publish(m, n, 0, colrow, tid);
     __syncthreads();
@@ -248,8 +248,6 @@ void c3_attributes() {
     std::call_once(once, [] {
         cudaFuncSetAttribute(k_coarse3d<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)kC3Smem);
-        cudaFuncSetAttribute(k_c3_setup<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             64 * (int)sizeof(double) * s2_pad(64));
     });
 }
 
@@ -281,7 +279,7 @@ void coarse3d_prepare() {
 
 template <typename T>
 bool coarse3d_plan(const MGHier<T>& H, int l0, C3Plan& P) {
-    return c3_plan<T>(H, l0, kC3Smem, sizeof(T) == 4 ? 64 : 27, P);
+    return c3_plan<T>(H, l0, kC3Smem, 27, P);
 }
 template <typename T>
 void coarse3d_sizes(const C3Plan& P, size_t* di, size_t* minv) {

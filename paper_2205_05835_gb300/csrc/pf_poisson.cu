@@ -69,6 +69,23 @@ template <typename T, int DIM>
 __device__ __forceinline__ void gs_cell(const MGLevel<T>& L, const T* __restrict__ phi,
                                         const Phys& ph, int i, int j, int k, int idx,
                                         bool zero_start) {
+    if constexpr (sizeof(T) == sizeof(double)) {
+        // (2 DIM + 2 float64 instructions instead of 4 DIM and a division: an SM has
+        // two float64 lanes)
+        if (L.di != nullptr) {
+            T s = T(0);
+            if (!zero_start) {
+                const Nb6 nb = nb6<DIM>(L.g, i, j, k, idx);
+#pragma unroll
+                for (int d = 0; d < DIM; ++d) {
+                    s += L.beta[d][idx] * L.x[nb.m[2 * d]];
+                    s += L.beta[d][nb.m[2 * d + 1]] * L.x[nb.m[2 * d + 1]];
+                }
+            }
+            L.x[idx] = (L.f[idx] + ih2_of(L.g, T()) * s) * L.di[idx];
+            return;
+        }
+    }
     const Nb6 nb = nb6<DIM>(L.g, i, j, k, idx);
     T w[6];
     face_w<T, DIM>(L, phi, ph, idx, nb, w);
@@ -221,6 +238,56 @@ k_gs(MGLevel<T> L, const T* __restrict__ phi, Phys ph, int cls, int zero_start,
                 gs_cell<T, DIM>(L, phi, ph, i, j, k, idx, false);
         });
     }
+}
+
+// inverse diagonals of a float64 level (once per solve)
+template <typename T, int DIM>
+__global__ void __launch_bounds__(kThreads)
+k_invdiag(MGLevel<T> L) {
+    const T ih2 = ih2_of(L.g, T());
+    for_cells(L.g, [&](int i, int j, int k, int idx) {
+        const Nb6 nb = nb6<DIM>(L.g, i, j, k, idx);
+        T d = T(0);
+#pragma unroll
+        for (int q = 0; q < DIM; ++q) d += L.beta[q][idx] + L.beta[q][nb.m[2 * q + 1]];
+        L.di[idx] = T(1) / (ih2 * d);
+    });
+}
+
+// The restriction of an even level after its sweeps, from the first colour
+// alone: the second colour's residual is zero, and after one sweep from zero
+// the first colour's is the neighbours' part.
+template <typename T, int DIM>
+__global__ void __launch_bounds__(kThreads)
+k_restrict_even(MGLevel<T> F, MGLevel<T> C, int one_sweep, const CGScalars* sc) {
+    if (inner_stopped(sc)) return;
+    const T ih2 = ih2_of(F.g, T());
+    for_cells(C.g, [&](int ci, int cj, int ck, int I) {
+        T s = T(0), fs = T(0);
+#pragma unroll
+        for (int a = 0; a < (DIM == 3 ? 2 : 1); ++a)
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+                const int fi = 2 * ci + ((a + b) & 1), fj = 2 * cj + b,
+                          fk = DIM == 3 ? 2 * ck + a : 0;
+                const int idx = (fk * F.g.ny + fj) * F.g.nx + fi;
+                const Nb6 nb = nb6<DIM>(F.g, fi, fj, fk, idx);
+                const T xc = one_sweep ? T(0) : F.x[idx];
+#pragma unroll
+                for (int d = 0; d < DIM; ++d) {
+                    const T b0 = F.beta[d][idx], b1 = F.beta[d][nb.m[2 * d + 1]];
+                    T x0 = F.x[nb.m[2 * d]], x1 = F.x[nb.m[2 * d + 1]];
+                    if (!one_sweep) {
+                        x0 -= xc;
+                        x1 -= xc;
+                    }
+                    s += b0 * x0;
+                    s += b1 * x1;
+                }
+                if (!one_sweep) fs += F.f[idx];
+            }
+        C.f[I] = (fs + ih2 * s) * T(DIM == 3 ? 0.125 : 0.25);
+    });
 }
 
 template <typename T, int DIM, bool UNI>
@@ -708,6 +775,9 @@ void launch_mg_setup(const Dims&, const Phys& ph, const T* phi, MGHier<T>& H, cu
         k_coarsen_beta<T, DIM><<<row_grid(H.lev[l + 1].g, kThreads, 1 << 30), kThreads, 0, s>>>(
             H.lev[l], H.lev[l + 1], phi, ph);
     }
+    for (int l = 0; l < H.first_coarse; ++l)
+        if (H.lev[l].di != nullptr)
+            k_invdiag<T, DIM><<<row_grid(H.lev[l].g, kThreads, 1 << 30), kThreads, 0, s>>>(H.lev[l]);
     if (DIM == 3 && use_coarse3d(H)) launch_coarse3d_setup<T>(*H.c3, H, s);
 }
 
@@ -792,7 +862,9 @@ T* launch_vcycle(const Phys& ph, const T* phi, MGHier<T>& H, const CGScalars* sc
         }
         if (!done_r) {
             const int gr = row_grid(H.lev[l + 1].g, kThreads, 1 << 30);
-            if (uniform_pair<T, DIM>(L, H.lev[l + 1]))
+            if (L.di != nullptr && uniform_pair<T, DIM>(L, H.lev[l + 1]) && gs_classes(L.g) == 2)
+                k_restrict_even<T, DIM><<<gr, kThreads, 0, s>>>(L, H.lev[l + 1], H.pre == 1, sc);
+            else if (uniform_pair<T, DIM>(L, H.lev[l + 1]))
                 k_restrict<T, DIM, true><<<gr, kThreads, 0, s>>>(L, H.lev[l + 1], phi, ph, sc);
             else
                 k_restrict<T, DIM, false><<<gr, kThreads, 0, s>>>(L, H.lev[l + 1], phi, ph, sc);

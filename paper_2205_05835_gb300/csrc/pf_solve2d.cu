@@ -360,7 +360,7 @@ __global__ void __launch_bounds__(kS2Threads, 1) k_solve2d(const __grid_constant
         __syncthreads();
         s2_dense_fill(S[ld], M, tid);
         __syncthreads();
-        T m[8];
+        T m[2];
         s2_gj_move(m, M, n, false, tid);
         s2_gj_publish(m, n, 0, colrow, tid);
         __syncthreads();
@@ -525,7 +525,7 @@ __global__ void __launch_bounds__(kS2Threads, 1) k_solve2d(const __grid_constant
 // kernels on the whole chip are faster: a mixed step of 640^2 takes 5.3 ms
 // here and 7.3 ms there, of 768^2 9.5 and 6.2 ms; a float64 one of 512^2 11.3
 // and 13.8 ms (larger ones do not fit).
-template <typename T> constexpr int kMaxCtaCells = sizeof(T) == 4 ? 27000 : 16500;
+template <typename T> constexpr int kMaxCtaCells = sizeof(T) == 4 ? 27000 : kSolve2dCells64 / 16;
 
 // dynamic shared memory left beside the kernel's static arrays
 template <typename T>
@@ -538,14 +538,12 @@ size_t dynamic_smem() {
 template <typename T>
 S2Limits limits(int max_cluster) {
     // Cycles measured at 64^2 .. 256^2: a phase of a cluster costs about 900
-    // beside its cells, one of a CTA 400. The inverse of 64 cells costs about
-    // 20k cycles a solve in float32, a float64 one of 16 cells as much. The
-    // fused interpolation has 31 instructions a cell instead of 4, too many for
+    // beside its cells, one of a CTA 400. The fused interpolation has 31 instructions a cell instead of 4, too many for
     // the float64 pipe.
     const bool f32 = sizeof(T) == 4;
     S2Limits m;
     m.max_cluster = max_cluster;
-    m.dense_cells = f32 ? 64 : 16;
+    m.dense_cells = f32 ? 27 : 16;
     m.fused_cells = f32 ? 2048 : 0;
     m.cta_cells = kMaxCtaCells<T>;
     m.cell = f32 ? 8.f : 28.f;

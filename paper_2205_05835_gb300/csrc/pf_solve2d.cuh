@@ -525,42 +525,40 @@ PF_HD void s2_dense_fill(const S2View<T>& L, T* M, int t) {
         }
     }
 }
-// Elimination: a thread keeps its eight elements (column t % 64, rows t / 64 +
-// 8 i) in registers; publish copies column k, row k and the pivot's reciprocal
-// of the current matrix into one of two buffers, step reads them. One barrier
-// a step.
-constexpr int kS2Col = 64, kS2ColRow = 129;   // offsets of the row; elements of a buffer
+// Elimination: a thread keeps its two elements (column t % 32, rows t / 32 and
+// t / 32 + 16) in registers; publish copies column k, row k and the pivot's
+// reciprocal of the current matrix into one of two buffers, step reads them.
+// One barrier a step. (64 cells took 45 us a solve, more than the level that
+// 16 to 27 cells add costs in ten V-cycles.)
+constexpr int kS2DenseMax = 32;                       // cells of a dense level
+constexpr int kS2Col = kS2DenseMax, kS2ColRow = 2 * kS2DenseMax + 1;   // the row's offset; size
 template <typename T>
-PF_HD void s2_gj_publish(const T (&m)[8], int n, int k, T* buf, int t) {
-    const int c = t & 63, r0 = t >> 6;
+PF_HD void s2_gj_publish(const T (&m)[2], int n, int k, T* buf, int t) {
+    const int c = t & 31, r0 = t >> 5;
     if (c >= n || k >= n) return;
     if (c == k) {
-        for (int i = 0; i < 8; ++i)
-            if (r0 + 8 * i < n) buf[r0 + 8 * i] = m[i];
+        if (r0 < n) buf[r0] = m[0];
+        if (r0 + 16 < n) buf[r0 + 16] = m[1];
     }
-    if (r0 == (k & 7)) {
-        T v = m[0];
-        for (int i = 1; i < 8; ++i) v = i == (k >> 3) ? m[i] : v;
+    if (r0 == (k & 15)) {
+        const T v = k < 16 ? m[0] : m[1];
         buf[kS2Col + c] = v;
-        if (c == k) buf[128] = T(1) / v;
+        if (c == k) buf[2 * kS2Col] = s2_rcp(v);
     }
 }
 template <typename T>
-PF_HD void s2_gj_step(T (&m)[8], int n, int k, const T* buf, int t) {
-    const int c = t & 63, r0 = t >> 6;
+PF_HD void s2_gj_step(T (&m)[2], int n, int k, const T* buf, int t) {
+    const int c = t & 31, r0 = t >> 5;
     if (c >= n) return;
-    const T rk = (c == k ? T(1) : buf[kS2Col + c]) * buf[128];
-    for (int i = 0; i < 8; ++i) {
-        const int r = r0 + 8 * i;
-        if (r >= n) continue;
-        m[i] = r == k ? rk : (c == k ? T(0) : m[i]) - buf[r] * rk;
-    }
+    const T rk = (c == k ? T(1) : buf[kS2Col + c]) * buf[2 * kS2Col];
+    if (r0 < n) m[0] = r0 == k ? rk : (c == k ? T(0) : m[0]) - buf[r0] * rk;
+    if (r0 + 16 < n) m[1] = r0 + 16 == k ? rk : (c == k ? T(0) : m[1]) - buf[r0 + 16] * rk;
 }
 template <typename T>
-PF_HD void s2_gj_move(T (&m)[8], T* M, int n, bool store, int t) {
-    const int c = t & 63, ld = s2_pad(n);
-    for (int i = 0; i < 8; ++i) {
-        const int r = (t >> 6) + 8 * i;
+PF_HD void s2_gj_move(T (&m)[2], T* M, int n, bool store, int t) {
+    const int c = t & 31, ld = s2_pad(n);
+    for (int i = 0; i < 2; ++i) {
+        const int r = (t >> 5) + 16 * i;
         if (c < n && r < n) {
             if (store) M[r * ld + c] = m[i];
             else m[i] = M[r * ld + c];
@@ -581,13 +579,13 @@ PF_HD void s2_dense_means(const T* M, int n, int k, T* colrow, int t) {
     const int ld = s2_pad(n);
     const T* d = colrow + kS2ColRow;
     T s = T(0), w = T(0);
-    if (k == 1 && (t < n || (t >= 64 && t < 64 + n))) {
+    if (k == 1 && (t < n || (t >= kS2Col && t < kS2Col + n))) {
         for (int c = 0; c < n; ++c) {
-            s += d[c] * (t < 64 ? M[t * ld + c] : M[c * ld + t - 64]);
+            s += d[c] * (t < kS2Col ? M[t * ld + c] : M[c * ld + t - kS2Col]);
             w += d[c];
         }
         colrow[t] = s / w;
-    } else if (k == 2 && t == 128) {
+    } else if (k == 2 && t == 2 * kS2Col) {
         for (int c = 0; c < n; ++c) {
             s += d[c] * colrow[c];
             w += d[c];
@@ -597,10 +595,10 @@ PF_HD void s2_dense_means(const T* M, int n, int k, T* colrow, int t) {
 }
 template <typename T>
 PF_HD void s2_dense_project(T* M, int n, const T* colrow, int t) {
-    const int ld = s2_pad(n), c = t & 63;
+    const int ld = s2_pad(n), c = t & 31;
     if (c < n)
-        for (int r = t >> 6; r < n; r += kS2Threads >> 6)
-            M[r * ld + c] -= (colrow[r] + colrow[64 + c]) - colrow[128];
+        for (int r = t >> 5; r < n; r += kS2Threads >> 5)
+            M[r * ld + c] -= (colrow[r] + colrow[kS2Col + c]) - colrow[2 * kS2Col];
 }
 // x = M f of the part of thread t: row t / 8, every eighth column from t % 8
 template <typename T>
@@ -613,7 +611,6 @@ PF_HD T s2_dense_part(const T* M, const T* f, int n, int t) {
     }
     return s;
 }
-constexpr int kS2DenseMax = kS2Threads / 8;   // cells of a dense level
 
 // Sums whose rounding is carried along: float64 sums of the float64 path,
 // (hi, lo) float pairs of the mixed one (a float64 accumulation without GB300's

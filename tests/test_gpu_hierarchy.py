@@ -94,3 +94,30 @@ def test_2d_solve_residual(pf, n, ratio, precision, sweeps):
     floor = 8.0 * eps * max(b.max() for b in beta) / g.h ** 2 * np.linalg.norm(x)
     assert status == 0 and iters <= 40
     assert np.linalg.norm(r) <= 1.01 * rtol * np.linalg.norm(rhs) + floor
+
+
+@pytest.mark.parametrize("n", [(32, 20, 12), (48, 32, 24), (24, 24, 24), (30, 22, 26)])
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("sweeps", [1, 2, 3])
+def test_3d_solve_residual(pf, n, precision, sweeps):
+    """The 3D hierarchy with several sweeps a level: the first-colour restriction
+    and inverse diagonals of the float64 levels, the cluster kernel below."""
+    rtol = 1e-10
+    p = I.small_case(dim=3, n=n[0], precision=precision, poisson_rtol=rtol, R=0.2,
+                     mg_pre=sweeps, mg_post=sweeps)
+    p["n"] = n
+    p = I.finalize(p)
+    po = O.params_from(p)
+    g = O.Grid(3, n, p["L"])
+    phi = O.initial_phi(po).astype(np.float32).astype(np.float64)
+    rhs = I.noise(g.shape, 6) - 0.5
+    rhs -= rhs.mean()
+    sim = pf.Simulation(p, phi0=phi)
+    x, iters, rel, status = sim.poisson_solve(rhs)
+    sim.close()
+    beta = O.face_beta(phi, g, po) if precision == "fp64" else beta32(phi, g, p)
+    r = rhs - O.apply_poisson(beta, x, g)
+    eps = 2.0 ** -47 if precision == "mixed" else 2.0 ** -52
+    floor = 12.0 * eps * max(b.max() for b in beta) / g.h ** 2 * np.linalg.norm(x)
+    assert status == 0 and iters <= 36
+    assert np.linalg.norm(r) <= 1.01 * rtol * np.linalg.norm(rhs) + floor
