@@ -286,72 +286,55 @@ inline int row_grid(const Dims& g, int threads, int cap) {
     return b < 1 ? 1 : (int)b;
 }
 
-// Sum of K values over the block (deterministic order). Result valid in thread 0.
+// Combines K values per thread over the block (deterministic order), through K
+// blockDim doubles of shared memory: warp k adds (mode 0) or maximises (mode 1)
+// value k, a few per lane, then over its lanes. A shuffle tree in every warp
+// would issue five times the float64 instructions, each of which occupies the
+// SM's two-lane float64 pipe for 19 cycles (with a maximum beside every sum
+// that was 90 of them a block: half of the 15 us of an update at 128^3).
+// Result valid in every thread.
 template <int K>
-__device__ __forceinline__ void block_reduce_sum(double (&v)[K], double* smem /* K*32 */) {
+__device__ __forceinline__ void block_combine(double (&v)[K], const int (&mode)[K], double* scr) {
+    const int nt = blockDim.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = nt >> 5;
 #pragma unroll
-    for (int q = 0; q < K; ++q)
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_down_sync(0xffffffffu, v[q], o);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    if (lane == 0)
-#pragma unroll
-        for (int q = 0; q < K; ++q) smem[q * 32 + warp] = v[q];
+    for (int k = 0; k < K; ++k) scr[k * nt + threadIdx.x] = v[k];
     __syncthreads();
-    if (warp == 0) {
 #pragma unroll
-        for (int q = 0; q < K; ++q) {
-            double t = lane < nw ? smem[q * 32 + lane] : 0.0;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-            v[q] = t;
+    for (int k = 0; k < K; ++k) {
+        if (warp != k % nw) continue;
+        double* p = scr + k * nt;
+        double t = p[lane];
+        for (int j = 1; j < nw; ++j) {
+            const double o = p[lane + 32 * j];
+            t = mode[k] == 0 ? t + o : fmax(t, o);
         }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const double u = __shfl_down_sync(0xffffffffu, t, o);
+            t = mode[k] == 0 ? t + u : fmax(t, u);
+        }
+        __syncwarp();
+        if (lane == 0) p[0] = t;
     }
     __syncthreads();
-}
-
-template <int K>
-__device__ __forceinline__ void block_reduce_max(double (&v)[K], double* smem) {
 #pragma unroll
-    for (int q = 0; q < K; ++q)
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v[q] = fmax(v[q], __shfl_down_sync(0xffffffffu, v[q], o));
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    if (lane == 0)
-#pragma unroll
-        for (int q = 0; q < K; ++q) smem[q * 32 + warp] = v[q];
-    __syncthreads();
-    if (warp == 0) {
-#pragma unroll
-        for (int q = 0; q < K; ++q) {
-            double t = lane < nw ? smem[q * 32 + lane] : -1.0e308;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) t = fmax(t, __shfl_down_sync(0xffffffffu, t, o));
-            v[q] = t;
-        }
-    }
+    for (int k = 0; k < K; ++k) v[k] = scr[k * nt];
     __syncthreads();
 }
 
 // Stores the block's K partials; returns true in every thread of the last
 // block to finish, after which `tot` holds the grid totals (fixed order).
 // Mode per value: 0 sum, 1 max. bid / nblocks: linear block index and count.
+// scr: K blockDim doubles of shared memory.
 template <int K>
 __device__ __forceinline__ bool grid_reduce_lin(double (&v)[K], const int (&mode)[K], RedBuf rb,
-                                                double (&tot)[K], int bid, int nblocks) {
-    __shared__ double smem[K * 32];
+                                                double (&tot)[K], int bid, int nblocks,
+                                                double* scr) {
     __shared__ bool last;
-    double s[K], m[K];
-#pragma unroll
-    for (int q = 0; q < K; ++q) {
-        s[q] = mode[q] == 0 ? v[q] : 0.0;
-        m[q] = mode[q] == 1 ? v[q] : -1.0e308;
-    }
-    block_reduce_sum<K>(s, smem);
-    block_reduce_max<K>(m, smem);
+    block_combine<K>(v, mode, scr);
     if (threadIdx.x == 0) {
 #pragma unroll
-        for (int q = 0; q < K; ++q) rb.part[bid * K + q] = mode[q] == 0 ? s[q] : m[q];
+        for (int q = 0; q < K; ++q) rb.part[bid * K + q] = v[q];
         __threadfence();
         unsigned t = atomicAdd(rb.counter, 1u);
         last = (t == (unsigned)nblocks - 1);
@@ -360,25 +343,24 @@ __device__ __forceinline__ bool grid_reduce_lin(double (&v)[K], const int (&mode
     if (!last) return false;
     __threadfence();
 #pragma unroll
-    for (int q = 0; q < K; ++q) {
-        s[q] = 0.0;
-        m[q] = -1.0e308;
-    }
+    for (int q = 0; q < K; ++q) tot[q] = mode[q] == 0 ? 0.0 : -1.0e308;
     for (int b = threadIdx.x; b < nblocks; b += blockDim.x) {
 #pragma unroll
         for (int q = 0; q < K; ++q) {
-            double t = __ldcg(rb.part + b * K + q);
-            if (mode[q] == 0) s[q] += t; else m[q] = fmax(m[q], t);
+            const double t = __ldcg(rb.part + b * K + q);
+            tot[q] = mode[q] == 0 ? tot[q] + t : fmax(tot[q], t);
         }
     }
-    block_reduce_sum<K>(s, smem);
-    block_reduce_max<K>(m, smem);
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int q = 0; q < K; ++q) tot[q] = mode[q] == 0 ? s[q] : m[q];
-        *rb.counter = 0u;
-    }
+    block_combine<K>(tot, mode, scr);
+    if (threadIdx.x == 0) *rb.counter = 0u;
     return true;
+}
+// the same for blocks of at most kThreads threads
+template <int K>
+__device__ __forceinline__ bool grid_reduce_lin(double (&v)[K], const int (&mode)[K], RedBuf rb,
+                                                double (&tot)[K], int bid, int nblocks) {
+    __shared__ double scr[K * kThreads];
+    return grid_reduce_lin<K>(v, mode, rb, tot, bid, nblocks, scr);
 }
 
 template <int K>

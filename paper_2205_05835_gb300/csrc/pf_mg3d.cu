@@ -347,11 +347,13 @@ __device__ __forceinline__ void sweep3d_body(const SweepArgs& A, unsigned char* 
     }
     cp_wait_all();
     if (A.dots) {
+        __syncthreads();   // the f ring is the reduction's scratch
         double v[2] = {double(rz), double(zq)}, tot[2];
         const int mode[2] = {0, 0};
         const int bid = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
         const int nb = gridDim.x * gridDim.y * gridDim.z;
-        if (grid_reduce_lin<2>(v, mode, A.rb, tot, bid, nb) && threadIdx.x == 0) {
+        if (grid_reduce_lin<2>(v, mode, A.rb, tot, bid, nb, reinterpret_cast<double*>(Fs)) &&
+            threadIdx.x == 0) {
             CGScalars* sc = A.scw;
             sc->beta = first_it ? 0.0 : -sc->alpha * tot[1] / sc->rz;
             sc->rz = tot[0];

@@ -413,7 +413,11 @@ k_sweep3d_tma(const __grid_constant__ CUtensorMap tm_rho, const __grid_constant_
         const int mode[2] = {0, 0};
         const int bid = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
         const int nb = gridDim.x * gridDim.y * gridDim.z;
-        if (grid_reduce_lin<2>(v, mode, A.rb, tot, bid, nb) && threadIdx.x == 0) {
+        // (the f ring, whose copies have landed, is the reduction's scratch)
+        static_assert(sizeof(S.f) >= 2 * C::NT * sizeof(double), "scratch");
+        if (grid_reduce_lin<2>(v, mode, A.rb, tot, bid, nb,
+                               reinterpret_cast<double*>(&S.f[0][0])) &&
+            threadIdx.x == 0) {
             CGScalars* scw = A.scw;
             scw->beta = first_it ? 0.0 : -scw->alpha * tot[1] / scw->rz;
             scw->rz = tot[0];
