@@ -1,6 +1,6 @@
 // The coarse part of a 3D V-cycle in one launch of a thread-block cluster: the
 // levels from about 32^3 cells down, each level's arrays in shared memory,
-// slabs of planes per CTA, the level of at most 27 cells solved
+// slabs of planes per CTA, the level of at most 32 cells solved
 // by its inverse. It replaces, per V-cycle, four launches per level of a few
 // thousand cells (4 to 5 us each) and a single-CTA kernel whose ~70 dependent
 // phases took 41 us at 16^3 in float32 and 118 us at 12^3 in float64.
@@ -279,7 +279,7 @@ void coarse3d_prepare() {
 
 template <typename T>
 bool coarse3d_plan(const MGHier<T>& H, int l0, C3Plan& P) {
-    return c3_plan<T>(H, l0, kC3Smem, 27, P);
+    return c3_plan<T>(H, l0, kC3Smem, kS2DenseMax, P);
 }
 template <typename T>
 void coarse3d_sizes(const C3Plan& P, size_t* di, size_t* minv) {

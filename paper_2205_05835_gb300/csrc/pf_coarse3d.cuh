@@ -148,11 +148,13 @@ PF_HD void c3_view_sizes(C3View<T>& v, const C3Lev& L, int k0, int np) {
     v.lh = s2_log2((L.nx + 1) >> 1);
     v.inv_ny = 1.0f / float(L.ny);
 }
-PF_HD int c3_bits(int s) { return (s & 1) + ((s >> 1) & 1) + ((s >> 2) & 1); }
 template <typename T>
-PF_HD int c3_classes(const C3View<T>& L) { return 2 + 2 * c3_bits(L.seams); }
-PF_HD int c3_seams(int s, int i, int j, int k, int nx, int ny, int nz) {
-    return ((s & 1) && i == nx - 1) + ((s & 2) && j == ny - 1) + ((s & 4) && k == nz - 1);
+PF_HD int c3_classes(const C3View<T>& L) { return L.seams ? 3 : 2; }
+// class of a cell of a level with an odd or one-cell axis (see s2_class)
+PF_HD int c3_class(int s, int i, int j, int k, int nx, int ny, int nz) {
+    const int a = ((s & 1) && i == nx - 1 ? 2 : (i & 1)) + ((s & 2) && j == ny - 1 ? 2 : (j & 1)) +
+                  ((s & 4) && k == nz - 1 ? 2 : (k & 1));
+    return a >= 6 ? 0 : (a >= 3 ? a - 3 : a);
 }
 
 // Loops over the rows (r: plane, j) of a slab and n items of a row. The plane
@@ -214,17 +216,24 @@ PF_HD void c3_start(const C3View<T>& L, int r, int j, int i, int idx, T f) {
     if (!L.seams) {
         if (c0) L.x[idx] = f * L.di[idx];
     } else {
-        L.x[idx] = c0 && c3_seams(L.seams, i, j, k, L.nx, L.ny, L.nz) == 0 ? f * L.di[idx] : T(0);
+        L.x[idx] = c3_class(L.seams, i, j, k, L.nx, L.ny, L.nz) == 0 ? f * L.di[idx] : T(0);
     }
 }
 
 template <typename T>
 PF_HD void c3_gs(const C3View<T>& L, int cls, int t) {
-    const int nx = L.nx, color = cls & 1, want = cls >> 1;
-    c3_cells((nx + 1) >> 1, L.ny, L.np, L.inv_ny, L.lh, t, [&](int r, int j, int m) {
-        const int k = L.k0 + r, i = 2 * m + ((j + k + color) & 1);
+    const int nx = L.nx;
+    if (L.seams) {
+        c3_cells(nx, L.ny, L.np, L.inv_ny, L.lf, t, [&](int r, int j, int i) {
+            const int idx = (r * L.ny + j) * nx + i;
+            if (c3_class(L.seams, i, j, L.k0 + r, nx, L.ny, L.nz) == cls)
+                L.x[idx] = c3_off(L, r, j, i, idx, L.f[idx]) * L.di[idx];
+        });
+        return;
+    }
+    c3_cells(nx >> 1, L.ny, L.np, L.inv_ny, L.lh, t, [&](int r, int j, int m) {
+        const int i = 2 * m + ((j + L.k0 + r + cls) & 1);
         const int idx = (r * L.ny + j) * nx + i;
-        if (L.seams && (i >= nx || c3_seams(L.seams, i, j, k, nx, L.ny, L.nz) != want)) return;
         L.x[idx] = c3_off(L, r, j, i, idx, L.f[idx]) * L.di[idx];
     });
 }

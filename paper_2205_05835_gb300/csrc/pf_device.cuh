@@ -224,17 +224,20 @@ __device__ __forceinline__ void for_cells(const Dims& g, F f) {
     }
 }
 
-// Classes of a Gauss-Seidel sweep on a periodic level: colour (i + j + k) % 2
-// plus 2 s, s the number of axes of odd size along which the cell is the last
-// one. Two neighbours never share a class: across an odd axis's seam, where
-// their colours agree, s differs by one. Even levels have the two colours only.
+// Classes of a Gauss-Seidel sweep on a periodic level: the colours (i + j + k) % 2
+// where every axis is even; else the sum modulo 3 of a value per axis that
+// alternates 0, 1 and is 2 on the last cell of an odd axis. Two neighbours never
+// share a class, across an odd axis's seam either.
 __host__ __device__ __forceinline__ int odd_axis(int n) { return n > 1 ? (n & 1) : 0; }
-__host__ __device__ __forceinline__ int gs_classes(const Dims& g) {
-    return 2 + 2 * (odd_axis(g.nx) + odd_axis(g.ny) + odd_axis(g.nz));
+__host__ __device__ __forceinline__ bool gs_odd(const Dims& g) {
+    return odd_axis(g.nx) || odd_axis(g.ny) || odd_axis(g.nz);
 }
-__device__ __forceinline__ int gs_seams(const Dims& g, int i, int j, int k) {
-    return (odd_axis(g.nx) && i == g.nx - 1) + (odd_axis(g.ny) && j == g.ny - 1) +
-           (odd_axis(g.nz) && k == g.nz - 1);
+__host__ __device__ __forceinline__ int gs_classes(const Dims& g) { return gs_odd(g) ? 3 : 2; }
+__device__ __forceinline__ int gs_class(const Dims& g, int i, int j, int k) {
+    const int a = (odd_axis(g.nx) && i == g.nx - 1 ? 2 : (i & 1)) +
+                  (odd_axis(g.ny) && j == g.ny - 1 ? 2 : (j & 1)) +
+                  (odd_axis(g.nz) && k == g.nz - 1 ? 2 : (k & 1));
+    return a >= 6 ? 0 : (a >= 3 ? a - 3 : a);
 }
 
 // Same, over the cells of one colour ((i + j + k) % 2 == color).

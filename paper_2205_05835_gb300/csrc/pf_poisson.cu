@@ -223,19 +223,22 @@ __global__ void __launch_bounds__(kThreads)
 k_gs(MGLevel<T> L, const T* __restrict__ phi, Phys ph, int cls, int zero_start,
      const CGScalars* sc) {
     if (inner_stopped(sc)) return;
-    const int color = cls & 1, seams = cls >> 1;
-    const bool odd = gs_classes(L.g) > 2;
+    const bool odd = gs_odd(L.g);
     if (zero_start) {
         // every class: the active one x = f/diag, the others 0
         for_cells(L.g, [&](int i, int j, int k, int idx) {
-            if (((i + j + k) & 1) == color && (!odd || gs_seams(L.g, i, j, k) == seams))
+            if ((odd ? gs_class(L.g, i, j, k) : ((i + j + k) & 1)) == cls)
                 gs_cell<T, DIM>(L, phi, ph, i, j, k, idx, true);
             else L.x[idx] = T(0);
         });
-    } else {
-        for_color_cells(L.g, color, [&](int i, int j, int k, int idx) {
-            if (!odd || gs_seams(L.g, i, j, k) == seams)
+    } else if (odd) {
+        for_cells(L.g, [&](int i, int j, int k, int idx) {
+            if (gs_class(L.g, i, j, k) == cls)
                 gs_cell<T, DIM>(L, phi, ph, i, j, k, idx, false);
+        });
+    } else {
+        for_color_cells(L.g, cls, [&](int i, int j, int k, int idx) {
+            gs_cell<T, DIM>(L, phi, ph, i, j, k, idx, false);
         });
     }
 }
@@ -567,8 +570,18 @@ template <typename T, int DIM>
 __device__ __forceinline__ void cta_cells(const Dims& g, int cls, bool all, const MGLevel<T>& L,
                                           const T* phi, const Phys& ph, bool zero_start,
                                           int t0, int nt) {
-    const int color = cls & 1, seams = cls >> 1;
-    const bool odd = gs_classes(g) > 2;
+    if (gs_odd(g)) {
+        const float inv_nx = 1.0f / float(g.nx), inv_ny = 1.0f / float(g.ny);
+        for (int q = t0; q < g.ncell; q += nt) {
+            const int r = int((float(q) + 0.5f) * inv_nx), i = q - r * g.nx;
+            const int k = int((float(r) + 0.5f) * inv_ny), j = r - k * g.ny;
+            if (gs_class(g, i, j, k) == cls)
+                gs_cell<T, DIM>(L, phi, ph, i, j, k, q, zero_start);
+            else if (all) L.x[q] = T(0);
+        }
+        return;
+    }
+    const int color = cls;
     const int nhx = (g.nx + 1) >> 1;
     const int rows = g.ny * g.nz;
     const int items = rows * nhx;
@@ -581,11 +594,7 @@ __device__ __forceinline__ void cta_cells(const Dims& g, int cls, bool all, cons
         const int par = (j + k + color) & 1;
         const int i = 2 * m + par;
         const int base = r * g.nx;
-        if (i < g.nx) {
-            if (!odd || gs_seams(g, i, j, k) == seams)
-                gs_cell<T, DIM>(L, phi, ph, i, j, k, base + i, zero_start);
-            else if (all) L.x[base + i] = T(0);
-        }
+        if (i < g.nx) gs_cell<T, DIM>(L, phi, ph, i, j, k, base + i, zero_start);
         if (all) {
             const int io = 2 * m + (1 - par);
             if (io < g.nx) L.x[base + io] = T(0);

@@ -543,7 +543,7 @@ S2Limits limits(int max_cluster) {
     const bool f32 = sizeof(T) == 4;
     S2Limits m;
     m.max_cluster = max_cluster;
-    m.dense_cells = f32 ? 27 : 16;
+    m.dense_cells = f32 ? kS2DenseMax : 16;
     m.fused_cells = f32 ? 2048 : 0;
     m.cta_cells = kMaxCtaCells<T>;
     m.cell = f32 ? 8.f : 28.f;

@@ -193,7 +193,7 @@ PF_HD void s2_view_sizes(S2View<T>& v, const S2Lev& L, int j0, int rows) {
     v.qy = L.qy;
 }
 template <typename T>
-PF_HD int s2_classes(const S2View<T>& L) { return 2 + 2 * ((L.seams & 1) + ((L.seams >> 1) & 1)); }
+PF_HD int s2_classes(const S2View<T>& L) { return L.seams ? 3 : 2; }
 
 // Loops of a CTA's threads over its cells (f(r, i)) or pairs (2m, 2m + 1) of
 // cells of a row (f(r, m)): powers of two of threads along a row, so no thread
@@ -306,8 +306,14 @@ PF_HD void s2_coarsen(const S2View<T>& F, const S2View<T>& C, int t) {
     });
 }
 
-PF_HD int s2_seams(int seams, int i, int j, int nx, int ny) {
-    return ((seams & 1) && i == nx - 1) + ((seams & 2) && j == ny - 1);
+// Classes of the cells of a level with an odd or one-cell axis: the sum modulo 3
+// of a value per axis that alternates 0, 1 and is 2 on the last cell of an odd
+// axis, so two neighbours never share a class (three phases a sweep, where
+// colours with the seams' cells apart take four to six).
+PF_HD int s2_class(int seams, int i, int j, int nx, int ny) {
+    const int a = ((seams & 1) && i == nx - 1 ? 2 : (i & 1)) +
+                  ((seams & 2) && j == ny - 1 ? 2 : (j & 1));
+    return a >= 3 ? a - 3 : a;
 }
 
 // The first class of a sweep from zero, done where the right-hand side f of a
@@ -320,7 +326,7 @@ PF_HD void s2_start(const S2View<T>& L, int i, int j, int idx, T f) {
     if (!L.seams) {
         if (c0) L.x[idx] = f * L.di[idx];
     } else {
-        L.x[idx] = c0 && s2_seams(L.seams, i, j, L.nx, L.ny) == 0 ? f * L.di[idx] : T(0);
+        L.x[idx] = s2_class(L.seams, i, j, L.nx, L.ny) == 0 ? f * L.di[idx] : T(0);
     }
 }
 
@@ -328,8 +334,8 @@ PF_HD void s2_start(const S2View<T>& L, int i, int j, int idx, T f) {
 template <typename T>
 PF_HD void s2_gs(const S2View<T>& L, int cls, int t) {
     const int nx = L.nx;
-    const int color = cls & 1, want = cls >> 1;
     if (!L.seams) {
+        const int color = cls;
         s2_map<T>(nx >> 1, L.rows, L.lh, t,
                   [&](int r, int m) {
                       const int i = 2 * m + ((L.j0 + r + color) & 1), idx = r * nx + i;
@@ -338,9 +344,9 @@ PF_HD void s2_gs(const S2View<T>& L, int cls, int t) {
                   [&](int r, int m, T v) { L.x[r * nx + 2 * m + ((L.j0 + r + color) & 1)] = v; });
         return;
     }
-    s2_cells((nx + 1) >> 1, L.rows, L.lh, t, [&](int r, int m) {
-        const int j = L.j0 + r, i = 2 * m + ((j + color) & 1), idx = r * nx + i;
-        if (i >= nx || s2_seams(L.seams, i, j, nx, L.ny) != want) return;
+    s2_cells(nx, L.rows, L.lf, t, [&](int r, int i) {
+        const int idx = r * nx + i;
+        if (s2_class(L.seams, i, L.j0 + r, nx, L.ny) != cls) return;
         L.x[idx] = s2_off(L, r, i, idx, L.f[idx]) * L.di[idx];
     });
 }
@@ -646,28 +652,33 @@ template <> struct S2AccOf<float> { using type = S2AccF; };
 template <typename T, typename A>
 PF_HD void s2_gs_dots(const S2View<T>& L, const T* qv, bool first, A& rz, A& zq, int t) {
     const int nx = L.nx;
-    s2_map<T>((nx + 1) >> 1, L.rows, L.lh, t, [&](int r, int m) {
-        const int j = L.j0 + r, par = j & 1, i = 2 * m + par, o = 2 * m + 1 - par;
-        T x = T(0);
-        if (i < nx) {
+    if (L.seams) {
+        s2_cells(nx, L.rows, L.lf, t, [&](int r, int i) {
             const int idx = r * nx + i;
             const T f = L.f[idx];
-            x = !L.seams || s2_seams(L.seams, i, j, nx, L.ny) == 0
-                    ? s2_off(L, r, i, idx, f) * L.di[idx] : L.x[idx];
+            T x = L.x[idx];
+            if (s2_class(L.seams, i, L.j0 + r, nx, L.ny) == 0) {
+                x = s2_off(L, r, i, idx, f) * L.di[idx];
+                L.x[idx] = x;
+            }
             rz.add_prod(f, x);
             if (!first) zq.add_prod(x, qv[idx]);
-        }
-        if (o < nx) {
-            const int idx = r * nx + o;
-            const T y = L.x[idx];
-            rz.add_prod(L.f[idx], y);
-            if (!first) zq.add_prod(y, qv[idx]);
+        });
+        return;
+    }
+    s2_map<T>(nx >> 1, L.rows, L.lh, t, [&](int r, int m) {
+        const int j = L.j0 + r, par = j & 1, i = 2 * m + par, o = 2 * m + 1 - par;
+        const int idx = r * nx + i, ido = r * nx + o;
+        const T f = L.f[idx], y = L.x[ido];
+        const T x = s2_off(L, r, i, idx, f) * L.di[idx];
+        rz.add_prod(f, x);
+        rz.add_prod(L.f[ido], y);
+        if (!first) {
+            zq.add_prod(x, qv[idx]);
+            zq.add_prod(y, qv[ido]);
         }
         return x;
-    }, [&](int r, int m, T x) {
-        const int i = 2 * m + ((L.j0 + r) & 1);
-        if (i < nx) L.x[r * nx + i] = x;
-    });
+    }, [&](int r, int m, T x) { L.x[r * nx + 2 * m + ((L.j0 + r) & 1)] = x; });
 }
 
 // p = z + beta p (first: p = z)
