@@ -486,6 +486,7 @@ struct ImplT final : Impl {
             H.lev[l].f = cv.take<T>(m);
             for (int d = 0; d < 3; ++d) H.lev[l].beta[d] = d < DIM ? cv.take<T>(m) : nullptr;
         }
+        H.s2s = DIM == 2 ? cv.take<T>(n) : nullptr;
         // inverse diagonals of the float64 levels outside the coarse kernel (2D:
         // grids beyond the one-launch solve)
         for (int l = 0; l < kMaxLevels; ++l) H.lev[l].di = nullptr;
@@ -518,6 +519,7 @@ struct ImplT final : Impl {
     // Layout of a pressure solve alone (phi plus the solver's vectors), used by
     // the allocation-free entry point; the stage fields stay unset.
     void carve_solver_only(Carver& cv) {
+        H.s2s = nullptr;
         for (int l = 0; l < kMaxLevels; ++l) H.lev[l].di = nullptr;
         const size_t n = g.ncell;
         phiN = cv.take<T>(n);

@@ -161,6 +161,7 @@ struct MGHier {
     const struct C3Plan* c3 = nullptr;
     T* c3_di = nullptr;
     T* c3_minv = nullptr;
+    T* s2s = nullptr;   // 2D: s = A z of the one-launch solve, where shared memory is short
     int nlev;
     int first_coarse;   // levels >= first_coarse are handled by one kernel
     int pre, post;

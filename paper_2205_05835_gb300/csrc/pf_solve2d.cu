@@ -33,7 +33,7 @@ struct S2Args {
     T* b0;          // face coefficients to leave in the workspace (may be null)
     T* b1;
     T *gx[2], *gf[2], *gw0[2], *gw1[2];   // workspace places of levels 0 and 1
-    T *gdi, *gp, *gq, *ge;
+    T *gdi, *gp, *gq, *ge, *gs;
     CGScalars* sc;
 };
 
@@ -56,13 +56,13 @@ template <typename A>
 struct S2Red;
 template <>
 struct S2Red<S2AccF> {
-    S2AccF warp[2][kS2Warps];
-    S2AccF part[2][2][kS2MaxCTAs];   // [buffer][value][CTA], written by every CTA of the cluster
+    S2AccF warp[3][kS2Warps];
+    S2AccF part[2][3][kS2MaxCTAs];   // [buffer][value][CTA], written by every CTA of the cluster
 };
 template <>
 struct S2Red<S2AccD> {
-    S2AccD all[2][kS2Threads];
-    S2AccD part[2][2][kS2MaxCTAs];
+    S2AccD all[3][kS2Threads];
+    S2AccD part[2][3][kS2MaxCTAs];
 };
 
 // K totals over the cluster, valid in lane 0 of warps 0 .. K - 1 of every CTA
@@ -122,7 +122,7 @@ __device__ __forceinline__ void cluster_totals(A (&v)[K], A& tot, S2Red<A>& R, i
 template <typename T>
 struct S2Scal {
     T alpha, beta;
-    double rz, zq, pq;
+    double zq, zs, pq;
     double ff, rr, rr0_in, eta2;
     int done, idone, iters, it_in, outer, status, capped;
 };
@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(kS2Threads, 1) k_solve2d(const __grid_constant
     __shared__ S2View<T> S[kMaxLevels];
     __shared__ S2Red<A> R;
     __shared__ S2Scal<T> sc;
-    __shared__ T *vp, *vpm, *vpp, *vq, *ve;
+    __shared__ T *vp, *vq, *ve, *vs;
     __shared__ T colrow[2 * kS2ColRow];
     const S2Plan& P = a.P;
     const int C = P.C, rank = cluster_rank(), tid = threadIdx.x;
@@ -292,8 +292,7 @@ __global__ void __launch_bounds__(kS2Threads, 1) k_solve2d(const __grid_constant
                 vp = own(P.op, a.gp);
                 vq = own(P.oq, a.gq);
                 ve = own(P.oe, a.ge);
-                vpm = up(P.op, a.gp);
-                vpp = dn(P.op, a.gp);
+                vs = own(P.os, a.gs);
             }
         }
     } else if (tid >= 32 && tid - 32 + lc <= ld) {
@@ -439,7 +438,6 @@ __global__ void __launch_bounds__(kS2Threads, 1) k_solve2d(const __grid_constant
             if (rank == 0) single_vcycle(S, lc, ld, P.pre, P.post, P.fused, M);
             cluster_sync(C);
             // up
-            A d[2] = {A{}, A{}}, tot{};
             for (int l = lc - 1; l >= 0; --l) {
                 const S2View<T>& L = V[l];
                 // one phase less where a thread has few cells (the interpolation is
@@ -451,35 +449,31 @@ __global__ void __launch_bounds__(kS2Threads, 1) k_solve2d(const __grid_constant
                 const int nc = s2_classes(L);
                 for (int s = 0; s < P.post; ++s)
                     for (int k = nc - 1 - (fused && s == 0 ? 1 : 0); k >= 0; --k) {
-                        if (l == 0 && s == P.post - 1 && k == 0) {
-                            s2_gs_dots(L, vq, first, d[0], d[1], tid);
-                        } else {
-                            s2_gs(L, k, tid);
-                            cluster_sync(C);
-                        }
+                        s2_gs(L, k, tid);
+                        cluster_sync(C);
                     }
             }
-            // flexible CG: beta = -z.q / (p.q) of the last direction (Polak-Ribiere:
-            // alpha q is the last change of r)
-            cluster_totals<2>(d, tot, R, C, rank, buf);
+            // flexible CG with one set of products: s = A z, beta = -z.q / (p.q) of
+            // the last direction (Polak-Ribiere: alpha q is the last change of r),
+            // q = s + beta q and, A being symmetric, the new p.q = z.s + beta (2 z.q +
+            // beta p.q); A p formed from p itself takes a phase and a reduction more
+            A d[3] = {A{}, A{}, A{}}, tot{};
+            s2_apply_dots(L0, vq, vs, first, d[0], d[1], d[2], tid);
+            cluster_totals<3>(d, tot, R, C, rank, buf);
             if (tid == 32) sc.zq = tot.value();
+            if (tid == 64) sc.zs = tot.value();
             __syncthreads();
             if (tid == 0) {
-                sc.rz = tot.value();
-                sc.beta = first ? T(0) : T(-sc.zq / sc.pq);
+                const double rz = tot.value();
+                const double beta = first ? 0.0 : -sc.zq / sc.pq;
+                const double pq = first ? sc.zs : sc.zs + beta * (2.0 * sc.zq + beta * sc.pq);
+                sc.beta = T(beta);
+                sc.alpha = T(pq != 0.0 ? rz / pq : 0.0);
+                sc.pq = pq;
             }
             __syncthreads();
-            s2_direction(L0, vp, sc.beta, first, tid);
-            cluster_sync(C);
-            A pq[1] = {A{}};
-            s2_apply(L0, vp, vpm, vpp, vq, pq[0], tid);
-            cluster_totals<1>(pq, tot, R, C, rank, buf);
-            if (tid == 0) {
-                sc.pq = tot.value();
-                sc.alpha = T(sc.pq != 0.0 ? sc.rz / sc.pq : 0.0);
-            }
-            __syncthreads();
-            A rr[1] = {acc_of(s2_update(L0, vp, vq, ve, sc.alpha, first, tid))};
+            A rr[1] = {
+                acc_of(s2_update(L0, vs, vp, vq, ve, sc.alpha, sc.beta, first, tid))};
             cluster_totals<1>(rr, tot, R, C, rank, buf);
             if (tid == 0) {
                 const double v = tot.value();
@@ -592,7 +586,7 @@ void solve2d_prepare() {
 template <typename T>
 bool solve2d_plan(const MGHier<T>& H, bool beta_global, S2Plan& P) {
     const int mc = max_cluster<T>();
-    return mc > 0 && s2_plan<T>(H, limits<T>(mc), beta_global, P);
+    return mc > 0 && s2_plan<T>(H, limits<T>(mc), beta_global, H.s2s != nullptr, P);
 }
 
 template <typename T>
@@ -616,6 +610,7 @@ cudaError_t launch_solve2d(const S2Plan& P, const Dims& g, const Phys& ph,
     a.gdi = io.p[1];   // the second direction buffer is not needed here
     a.gq = io.q;
     a.ge = io.e;
+    a.gs = H.s2s != nullptr ? H.s2s : H.lev[0].x;
     a.sc = sc;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(P.C);

@@ -39,7 +39,7 @@ struct S2Plan {
     int lc;            // first level held by CTA 0 alone
     int ld;            // dense level: solved by its inverse (lc <= ld)
     int pre, post;
-    int op, oq, oe;    // offsets of p, q, e (-1: workspace)
+    int op, oq, oe, os;   // offsets of p, q, e, s (-1: workspace)
     int om;            // the dense level's inverse, padded rows of s2_pad(cells)
     int elems;         // dynamic shared memory, elements
     unsigned fused;    // bit l: s2_prolong_gs on level l (the same in every CTA)
@@ -80,9 +80,11 @@ struct S2Limits {
 
 // Fits the solve of a hierarchy into a cluster's shared memory: false when it
 // does not (too large a grid: more than cta_cells cells a CTA). beta_global:
-// the face coefficients also exist in the workspace.
+// the face coefficients also exist in the workspace; s_global: so does a place
+// for s.
 template <typename T>
-inline bool s2_plan(const MGHier<T>& H, const S2Limits& lim, bool beta_global, S2Plan& P) {
+inline bool s2_plan(const MGHier<T>& H, const S2Limits& lim, bool beta_global, bool s_global,
+                    S2Plan& P) {
     if (H.nlev < 2 || H.lev[0].g.nz != 1) return false;
     P.pre = H.pre;
     P.post = H.post;
@@ -143,8 +145,9 @@ inline bool s2_plan(const MGHier<T>& H, const S2Limits& lim, bool beta_global, S
     // level 0, in the order of use
     S2Lev& L = P.lev[0];
     const long long n0 = (long long)s2_max_rows(P, 0) * L.nx;
-    int* slots[8] = {&L.ox, &L.ow0, &L.ow1, &L.of, &L.od, &P.op, &P.oq, &P.oe};
-    for (int s = 0; s < 8; ++s) fits(slots[s], n0);
+    int* slots[9] = {&L.ox, &L.ow0, &L.ow1, &L.of, &L.od, &P.os, &P.oq, &P.op, &P.oe};
+    for (int s = 0; s < 9; ++s) fits(slots[s], n0);
+    if (P.os < 0 && !s_global && L.ox < 0) return false;   // (x's workspace place is free)
     P.fused = 0;
     for (int l = 0; l < P.ld; ++l) {
         const S2Lev &F = P.lev[l], &N = P.lev[l + 1];
@@ -647,88 +650,50 @@ struct S2AccD {
 template <typename T> struct S2AccOf { using type = S2AccD; };
 template <> struct S2AccOf<float> { using type = S2AccF; };
 
-// The last class (0) of the last post-sweep of level 0 with the CG products
-// rz = f.x and, unless first, zq = x.q over every cell of the strip.
+// s = A z (z: the level's x) and the products z.r, z.s and, unless first, z.q.
 template <typename T, typename A>
-PF_HD void s2_gs_dots(const S2View<T>& L, const T* qv, bool first, A& rz, A& zq, int t) {
-    const int nx = L.nx;
-    if (L.seams) {
-        s2_cells(nx, L.rows, L.lf, t, [&](int r, int i) {
-            const int idx = r * nx + i;
-            const T f = L.f[idx];
-            T x = L.x[idx];
-            if (s2_class(L.seams, i, L.j0 + r, nx, L.ny) == 0) {
-                x = s2_off(L, r, i, idx, f) * L.di[idx];
-                L.x[idx] = x;
-            }
-            rz.add_prod(f, x);
-            if (!first) zq.add_prod(x, qv[idx]);
-        });
-        return;
-    }
-    s2_map<T>(nx >> 1, L.rows, L.lh, t, [&](int r, int m) {
-        const int j = L.j0 + r, par = j & 1, i = 2 * m + par, o = 2 * m + 1 - par;
-        const int idx = r * nx + i, ido = r * nx + o;
-        const T f = L.f[idx], y = L.x[ido];
-        const T x = s2_off(L, r, i, idx, f) * L.di[idx];
-        rz.add_prod(f, x);
-        rz.add_prod(L.f[ido], y);
-        if (!first) {
-            zq.add_prod(x, qv[idx]);
-            zq.add_prod(y, qv[ido]);
-        }
-        return x;
-    }, [&](int r, int m, T x) { L.x[r * nx + 2 * m + ((L.j0 + r) & 1)] = x; });
-}
-
-// p = z + beta p (first: p = z)
-template <typename T>
-PF_HD void s2_direction(const S2View<T>& L, T* p, T beta, bool first, int t) {
-    s2_map<T>(L.nx, L.rows, L.lf, t, [&](int r, int i) {
-        const int k = r * L.nx + i;
-        return first ? L.x[k] : L.x[k] + beta * p[k];
-    }, [&](int r, int i, T v) { p[r * L.nx + i] = v; });
-}
-
-// q = A p and p.q; pm, pp: the rows of p around the strip
-template <typename T, typename A>
-PF_HD void s2_apply(const S2View<T>& L, const T* p, const T* pm, const T* pp, T* qv, A& pq, int t) {
+PF_HD void s2_apply_dots(const S2View<T>& L, const T* qv, T* sv, bool first, A& rz, A& zq, A& zs,
+                         int t) {
     const int nx = L.nx;
     s2_map<T>(nx, L.rows, L.lf, t, [&](int r, int i) {
         const int q = r * nx + i;
-        const int il = i == 0 ? q + nx - 1 : q - 1;
-        const int ir = i == nx - 1 ? q - i : q + 1;
-        const bool last = r == L.rows - 1;
-        const T* pu = r == 0 ? pm + i : p + (q - nx);
-        const T* pd = last ? pp + i : p + (q + nx);
-        const T* wd = last ? L.w1p + i : L.w1 + (q + nx);
-        const T pc = p[q], w0 = L.w0[q], wr = L.w0[ir], w1 = L.w1[q], w3 = *wd;
-        const T xl = p[il], xr = p[ir], xu = *pu, xd = *pd;
-        T ax = w0 * (pc - xl);
-        ax += wr * (pc - xr);
-        ax += w1 * (pc - xu);
-        ax += w3 * (pc - xd);
-        pq.add_prod(pc, ax);
+        const S2Nb<T> n = s2_nb(L, r, i, q);
+        const T z = L.x[q], w0 = L.w0[q], wr = L.w0[n.ir], w1 = L.w1[q], w3 = *n.wd;
+        const T xl = L.x[n.il], xr = L.x[n.ir], xu = *n.xu, xd = *n.xd;
+        T ax = w0 * (z - xl);
+        ax += wr * (z - xr);
+        ax += w1 * (z - xu);
+        ax += w3 * (z - xd);
+        rz.add_prod(z, L.f[q]);
+        zs.add_prod(z, ax);
+        if (!first) zq.add_prod(z, qv[q]);
         return ax;
-    }, [&](int r, int i, T v) { qv[r * nx + i] = v; });
+    }, [&](int r, int i, T v) { sv[r * nx + i] = v; });
 }
 
-// e += alpha p, r -= alpha q (r: the level's f), the next sweep's start;
-// per-thread sum of r^2
+// p = z + beta p, q = s + beta q, e += alpha p, r -= alpha q (r: the level's
+// f), the next sweep's start; per-thread sum of r^2.
 template <typename T>
-PF_HD T s2_update(const S2View<T>& L, const T* p, const T* qv, T* e, T alpha, bool first, int t) {
+PF_HD T s2_update(const S2View<T>& L, const T* sv, T* p, T* qv, T* e, T alpha, T beta, bool first,
+                  int t) {
     const int nx = L.nx;
     T rr = T(0);
-    struct ER { T e, r; };
-    s2_map<ER>(nx, L.rows, L.lf, t, [&](int r, int i) {
+    s2_cells(nx, L.rows, L.lf, t, [&](int r, int i) {
         const int k = r * nx + i;
-        return ER{first ? alpha * p[k] : e[k] + alpha * p[k], L.f[k] - alpha * qv[k]};
-    }, [&](int r, int i, ER v) {
-        const int k = r * nx + i;
-        e[k] = v.e;
-        L.f[k] = v.r;
-        s2_start(L, i, L.j0 + r, k, v.r);
-        rr += v.r * v.r;
+        const T z = L.x[k], s = sv[k], f = L.f[k];
+        T pn = z, qn = s, en = T(0);
+        if (!first) {
+            pn += beta * p[k];
+            qn += beta * qv[k];
+            en = e[k];
+        }
+        const T rv = f - alpha * qn;
+        p[k] = pn;
+        qv[k] = qn;
+        e[k] = en + alpha * pn;
+        L.f[k] = rv;
+        s2_start(L, i, L.j0 + r, k, rv);
+        rr += rv * rv;
     });
     return rr;
 }
