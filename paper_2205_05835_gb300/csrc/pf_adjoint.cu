@@ -16,9 +16,11 @@ namespace pf {
 
 namespace {
 
-__device__ __forceinline__ double clip01(double v) { return v < 0.0 ? 0.0 : (v > 1.0 ? 1.0 : v); }
-// d clip(phi) / d phi: 1 strictly inside (0, 1), 0 elsewhere
-__device__ __forceinline__ double dclip(double v) { return (v > 0.0 && v < 1.0) ? 1.0 : 0.0; }
+// d clip(phi) / d phi: 1 strictly inside (0, 1), 0 elsewhere (by the bits, as clip01)
+__device__ __forceinline__ double dclip(double v) {
+    const long long b = __double_as_longlong(v);
+    return b > 0 && b < 0x3ff0000000000000ll ? 1.0 : 0.0;
+}
 __device__ __forceinline__ double rho_c(double phi, const Phys& ph) {
     return ph.rho_out + ph.drho * clip01(phi);
 }

@@ -490,7 +490,7 @@ struct ImplT final : Impl {
         // inverse diagonals of the float64 levels outside the coarse kernel (2D:
         // grids beyond the one-launch solve)
         for (int l = 0; l < kMaxLevels; ++l) H.lev[l].di = nullptr;
-        if (sizeof(T) == sizeof(double) && (DIM == 3 || n > (size_t)kSolve2dCells64))
+        if (sizeof(T) == sizeof(double) && (DIM == 3 || n > (size_t)kSolve2dCells))
             for (int l = 0; l < H.first_coarse; ++l) H.lev[l].di = cv.take<T>(H.lev[l].g.ncell);
         // second buffers for the one-pass out-of-place sweeps (3D float32 levels
         // below the single-CTA levels)

@@ -100,11 +100,24 @@ struct Nbr {
 template <typename T>
 __device__ __forceinline__ T ldg(const T* p, int i) { return __ldg(p + i); }
 
+// clip(phi, 0, 1), NaN kept. In float64 by the bits: a comparison would run on
+// the float64 pipe (two lanes an SM), and a float64 stage clips some 30 values
+// a cell.
+__device__ __forceinline__ float clip01(float phi) {
+    return phi < 0.f ? 0.f : (phi > 1.f ? 1.f : phi);
+}
+__device__ __forceinline__ double clip01(double phi) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(phi);
+    const unsigned long long inf = 0x7ff0000000000000ull, one = 0x3ff0000000000000ull;
+    const unsigned long long m = b & ~(1ull << 63);
+    if (m > inf) return phi;                              // NaN
+    if (b >> 63) return m == 0 ? phi : 0.0;               // negative (-0 kept)
+    return m > one ? 1.0 : phi;
+}
 // Density (linear in clip(phi, 0, 1), phi = 1 the drop).
 template <typename T>
 __device__ __forceinline__ T rho_of_p(T phi, const PC<T>& c) {
-    const T s = phi < T(0) ? T(0) : (phi > T(1) ? T(1) : phi);
-    return c.rho_out + c.drho * s;
+    return c.rho_out + c.drho * clip01(phi);
 }
 
 // 1 / rho_f of the face between two cells in float32: a correctly rounded

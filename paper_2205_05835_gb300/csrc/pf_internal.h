@@ -402,7 +402,7 @@ void launch_coarse3d(const C3Plan& P, const MGHier<T>& H, const CGScalars* sc, c
 // solve2d_plan: false when the grid does not fit (use the kernels above).
 // b0, b1: the face coefficients of level 0, written (null: none are kept).
 struct S2Plan;
-constexpr int kSolve2dCells64 = 16 * 16500;   // float64 grids above do not take it
+constexpr int kSolve2dCells = 16 * 16500;   // larger grids do not take it
 void solve2d_prepare();
 template <typename T>
 bool solve2d_plan(const MGHier<T>& H, bool beta_global, S2Plan& P);

@@ -302,10 +302,18 @@ k_restrict(MGLevel<T> F, MGLevel<T> C, const T* __restrict__ phi, Phys ph, const
     });
 }
 
+// On an even level only the first colour: the post-sweep starts by overwriting
+// the second.
 template <typename T, int DIM, bool UNI>
 __global__ void __launch_bounds__(kThreads)
 k_prolong(MGLevel<T> F, MGLevel<T> C, const CGScalars* sc) {
     if (inner_stopped(sc)) return;
+    if (!gs_odd(F.g)) {
+        for_color_cells(F.g, 0, [&](int i, int j, int k, int idx) {
+            prolong_cell<T, DIM, UNI>(F, C, i, j, k, idx);
+        });
+        return;
+    }
     for_cells(F.g, [&](int i, int j, int k, int idx) {
         prolong_cell<T, DIM, UNI>(F, C, i, j, k, idx);
     });

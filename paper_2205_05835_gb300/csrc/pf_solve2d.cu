@@ -516,10 +516,10 @@ __global__ void __launch_bounds__(kS2Threads, 1) k_solve2d(const __grid_constant
 }
 
 // Largest strip (cells of level 0 per CTA) the cluster takes. Beyond it the
-// kernels on the whole chip are faster: a mixed step of 640^2 takes 5.3 ms
-// here and 7.3 ms there, of 768^2 9.5 and 6.2 ms; a float64 one of 512^2 11.3
-// and 13.8 ms (larger ones do not fit).
-template <typename T> constexpr int kMaxCtaCells = sizeof(T) == 4 ? 27000 : kSolve2dCells64 / 16;
+// kernels on the whole chip are faster: a mixed step of 512^2 takes 3.7 ms
+// here and 4.5 ms there, of 576^2 7.6 and 4.7 ms; a float64 one of 512^2 10.2
+// and 11.0 ms (larger ones do not fit).
+constexpr int kMaxCtaCells = kSolve2dCells / kS2MaxCTAs;
 
 // dynamic shared memory left beside the kernel's static arrays
 template <typename T>
@@ -539,7 +539,7 @@ S2Limits limits(int max_cluster) {
     m.max_cluster = max_cluster;
     m.dense_cells = f32 ? kS2DenseMax : 16;
     m.fused_cells = f32 ? 2048 : 0;
-    m.cta_cells = kMaxCtaCells<T>;
+    m.cta_cells = kMaxCtaCells;
     m.cell = f32 ? 8.f : 28.f;
     m.single_cell = f32 ? 5.f : 13.f;
     m.phase = 900.f;

@@ -14,16 +14,23 @@
 namespace pf {
 
 template <typename T>
-__device__ __forceinline__ T clamp01(T v) { return v < T(0) ? T(0) : (v > T(1) ? T(1) : v); }
-
-template <typename T>
 __device__ __forceinline__ T rho_of(T phi, const PC<T>& c) {
     return rho_of_p(phi, c);
 }
 
 template <typename T>
 __device__ __forceinline__ T eta_of(T phi, const PC<T>& c) {
-    return c.mu_out + c.dmu * clamp01(phi);
+    return c.mu_out + c.dmu * clip01(phi);
+}
+
+// the mean viscosity of four cells. Float64: one multiply-add on the sum of the
+// clipped values (the kernels are bound by the number of float64 instructions)
+template <typename T>
+__device__ __forceinline__ T eta_mean4(T a, T b, T c, T d, const PC<T>& q) {
+    if constexpr (sizeof(T) == sizeof(double))
+        return q.mu_out + (T(0.25) * q.dmu) * ((clip01(a) + clip01(b)) + (clip01(c) + clip01(d)));
+    else
+        return T(0.25) * (eta_of(a, q) + eta_of(b, q) + eta_of(c, q) + eta_of(d, q));
 }
 
 // velocity from the momentum rho_f u on the face between cells a and b
@@ -328,8 +335,11 @@ k_stage(Dims g, Phys ph, StageIO<T> io, int stage, int scheme, T wdt, T cdt, int
                     vel = T(0.25) * (ldg(ue, idx) + ldg(ue, nb.axc(e, e, 1)) + ldg(ue, im) +
                                      ldg(ue, nb.ax2c(e, d, -1, e, 1)));
                 }
-                adv = adv + vel * ((ldg(ud, nb.axc(d, e, 1)) - ldg(ud, nb.axc(d, e, -1))) * inv2h);
+                const T du = ldg(ud, nb.axc(d, e, 1)) - ldg(ud, nb.axc(d, e, -1));
+                if constexpr (sizeof(T) == sizeof(double)) adv = adv + vel * du;
+                else adv = adv + vel * (du * inv2h);
             }
+            if constexpr (sizeof(T) == sizeof(double)) adv = adv * inv2h;
         } else {
             // consistent transport: div(m u_d) in flux form, m the mass flux
             // rho_out u + (rho_in - rho_out) F of the CDI phase-field flux F
@@ -376,7 +386,23 @@ k_stage(Dims g, Phys ph, StageIO<T> io, int stage, int scheme, T wdt, T cdt, int
         const T etac = eta_of(pc, pcs), etam = eta_of(pm, pcs);
 #pragma unroll
         for (int e = 0; e < DIM; ++e) {
-            if (e == d) {
+            if constexpr (sizeof(T) == sizeof(double)) {
+                // the factors 1/h of the stresses and of their divergence once, below
+                if (e == d) {
+                    visc = visc + T(2) * (etac * (ldg(ud, nb.axc(d, d, 1)) - udc) -
+                                          etam * (udc - ldg(ud, im)));
+                } else {
+                    const T* __restrict__ ue = io.u_s[e];
+                    const int iep = nb.ax(e, 1), iepm = nb.ax2(d, -1, e, 1);
+                    const T eta_lo = eta_mean4(pc, pm, ldg(phi, nb.ax(e, -1)),
+                                               ldg(phi, nb.ax2(d, -1, e, -1)), pcs);
+                    const T eta_hi = eta_mean4(ldg(phi, iep), ldg(phi, iepm), pc, pm, pcs);
+                    const T slo = (udc - ldg(ud, nb.axc(d, e, -1))) + (ldg(ue, idx) - ldg(ue, im));
+                    const T shi = (ldg(ud, nb.axc(d, e, 1)) - udc) +
+                                  (ldg(ue, nb.axc(e, e, 1)) - ldg(ue, nb.ax2c(e, d, -1, e, 1)));
+                    visc = visc + (eta_hi * shi - eta_lo * slo);
+                }
+            } else if (e == d) {
                 T thi = T(2) * etac * ((ldg(ud, nb.axc(d, d, 1)) - udc) * inv_h);
                 T tlo = T(2) * etam * ((udc - ldg(ud, im)) * inv_h);
                 visc = visc + (thi - tlo) * inv_h;
@@ -397,6 +423,7 @@ k_stage(Dims g, Phys ph, StageIO<T> io, int stage, int scheme, T wdt, T cdt, int
                 visc = visc + (thi - tlo) * inv_h;
             }
         }
+        if constexpr (sizeof(T) == sizeof(double)) visc = visc * inv_h2;
         // surface tension force at the face
         const T dphi = (pc - pm) * inv_h;
         T F;
@@ -413,7 +440,8 @@ k_stage(Dims g, Phys ph, StageIO<T> io, int stage, int scheme, T wdt, T cdt, int
         }
         if (ph.momentum == 0) {
             const T beta = divq(T(1), T(0.5) * (rho_of(pc, pcs) + rho_of(pm, pcs)));
-            ku[d] = -adv + beta * visc + beta * F;
+            if constexpr (sizeof(T) == sizeof(double)) ku[d] = beta * (visc + F) - adv;
+            else ku[d] = -adv + beta * visc + beta * F;
         } else {
             ku[d] = -adv + visc + F;   // d(rho_f u_d)/dt
         }
