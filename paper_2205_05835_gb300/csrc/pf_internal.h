@@ -227,7 +227,7 @@ bool restrict3d_ok(const Dims& fine);
 // rho != nullptr (finest level): weights 2 / (rho_c + rho_q) from the cell
 // densities instead of the level's face arrays.
 void launch_restrict3d(const MGLevel<float>& F, const MGLevel<float>& C, const float* rho,
-                       const CGScalars* sc, cudaStream_t s);
+                       bool one_sweep, const CGScalars* sc, cudaStream_t s);
 // The fused stage of the 3D float32 path (pf_stage_fused.cu): cell pass and
 // stage in one kernel for CDI / ACDI with the EB force and advective transport.
 bool stage_fused_ok(const Dims& g, const Phys& ph);

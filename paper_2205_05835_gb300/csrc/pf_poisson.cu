@@ -873,7 +873,7 @@ T* launch_vcycle(const Phys& ph, const T* phi, MGHier<T>& H, const CGScalars* sc
             if (L.beta[0] != nullptr && restrict3d_ok(L.g)) {
                 launch_restrict3d(reinterpret_cast<const MGLevel<float>&>(L),
                                   reinterpret_cast<const MGLevel<float>&>(H.lev[l + 1]),
-                                  l == 0 ? H.rho0 : H.rhoc[l], sc, s);
+                                  l == 0 ? H.rho0 : H.rhoc[l], H.pre == 1, sc, s);
                 done_r = true;
             }
         }

@@ -121,3 +121,34 @@ def test_3d_solve_residual(pf, n, precision, sweeps):
     floor = 12.0 * eps * max(b.max() for b in beta) / g.h ** 2 * np.linalg.norm(x)
     assert status == 0 and iters <= 36
     assert np.linalg.norm(r) <= 1.01 * rtol * np.linalg.norm(rhs) + floor
+
+
+@pytest.mark.parametrize("n", [(40, 24, 16), (72, 40, 24), (132, 36, 20), (68, 20, 140)])
+@pytest.mark.parametrize("ratio", [10.0, 1000.0])
+def test_3d_mixed_first_colour_restriction(pf, n, ratio):
+    """Column-marching restriction after one sweep from zero (first colour alone,
+    from densities and, below level 1, from face arrays), ragged column tiles and
+    several z chunks: against the one that reads every cell (two sweeps). A
+    V(2, 2) cycle does no more than two V(1, 1) cycles, so one sweep takes at
+    most twice its iterations (and one per refinement, of which there are two)."""
+    iters = {}
+    for sweeps in (1, 2):
+        p = I.small_case(dim=3, n=n[0], precision="mixed", poisson_rtol=1e-10, R=0.2,
+                         rho_in=10.0, rho_out=10.0 / ratio, mg_pre=sweeps, mg_post=sweeps,
+                         mg_coarse_cells=64)
+        p["n"] = n
+        p = I.finalize(p)
+        po = O.params_from(p)
+        g = O.Grid(3, n, p["L"])
+        phi = O.initial_phi(po).astype(np.float32).astype(np.float64)
+        rhs = I.noise(g.shape, 6) - 0.5
+        rhs -= rhs.mean()
+        sim = pf.Simulation(p, phi0=phi)
+        x, iters[sweeps], rel, status = sim.poisson_solve(rhs)
+        sim.close()
+        beta = beta32(phi, g, p)
+        r = rhs - O.apply_poisson(beta, x, g)
+        floor = 12.0 * 2.0 ** -47 * max(b.max() for b in beta) / g.h ** 2 * np.linalg.norm(x)
+        assert status == 0
+        assert np.linalg.norm(r) <= 1.01e-10 * np.linalg.norm(rhs) + floor
+    assert iters[1] <= 2 * iters[2] + 2
