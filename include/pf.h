@@ -120,8 +120,10 @@ typedef struct {
                              PF_SHAPE_WAVE (needs wall_y = 1): phi = 1 below the interface
                              y = R (1 - pert_amp cos(k (x - dx/2))), k = 2 pi pert_mode / (n[0] dx)
                              (R: mean height, pert_amp: amplitude over R) */
-    int mg_coarse_cells;  /* multigrid levels of at most this many cells are solved together by
-                             one single-CTA V-cycle kernel (0: 4096; else 16 .. 2^20). A
+    int mg_coarse_cells;  /* multigrid levels of at most this many cells (16 .. 2^20) are solved
+                             together by one coarse V-cycle launch. 0: in 3D the levels of
+                             at most 40000 cells that fit into the shared memory of a cluster,
+                             else 4096. 2D grids whose whole solve is one launch ignore it. A
                              tuning knob: it changes the preconditioner, not the converged
                              solution (see the package's autotune module) */
     int sweep_staging;    /* finest-level red-black sweeps of the 3D mixed path: 0 (default)

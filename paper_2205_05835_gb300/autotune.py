@@ -4,8 +4,9 @@ The tunables change the preconditioner of the pressure solve, never the
 converged answer (every candidate solves to the same poisson_rtol):
 
   mg_coarse_cells -- levels of at most this many cells are handled together
-                     by one single-CTA V-cycle launch (fewer, longer launches
-                     against more, shorter ones);
+                     by one coarse V-cycle launch (fewer, longer launches
+                     against more, shorter ones; 0: the library's rule; no
+                     effect on 2D grids whose whole solve is one launch);
   mg_pre, mg_post -- red-black sweeps before and after the coarse correction
                      (cheaper V-cycles against fewer CG iterations);
   sweep_tile      -- 3D mixed precision, tuned second with the best shape
@@ -35,11 +36,11 @@ import os
 import time
 
 CANDIDATES = tuple(
-    [{"mg_coarse_cells": c, "mg_pre": v, "mg_post": v} for v in (1, 2) for c in (1024, 4096, 16384)]
-    + [{"mg_coarse_cells": c, "mg_pre": v, "mg_post": v} for v in (3, 4, 6) for c in (4096, 16384)]
-    + [{"mg_coarse_cells": 4096, "mg_pre": v, "mg_post": v} for v in (8, 10)])
+    [{"mg_coarse_cells": c, "mg_pre": v, "mg_post": v} for v in (1, 2) for c in (1024, 0, 16384)]
+    + [{"mg_coarse_cells": c, "mg_pre": v, "mg_post": v} for v in (3, 4, 6) for c in (0, 16384)]
+    + [{"mg_coarse_cells": 0, "mg_pre": v, "mg_post": v} for v in (8, 10)])
 
-DEFAULT_SHAPE = {"mg_coarse_cells": 4096, "mg_pre": 1, "mg_post": 1}   # the library's defaults
+DEFAULT_SHAPE = {"mg_coarse_cells": 0, "mg_pre": 1, "mg_post": 1}   # the library's defaults
 MARGIN = 0.01                            # relative gain needed to leave a default
 
 INNER_TOLS = (1e-6, 1e-5, 1e-4, 1e-3)   # the first is the library's default
