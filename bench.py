@@ -256,10 +256,10 @@ FINEST_CLASSES = ("mg_gs_level0", "cg_dir_spmv", "cg_update", "ir_residual_f64",
 
 
 def mg_levels(n, dim, coarse_cells=4096):
-    """Cells of the tiled multigrid levels (those below the single-CTA coarse
-    solve), finest first, by the library's rule: a level has a coarser one
-    while every axis is even and at least 4; the first level of at most
-    `coarse_cells` cells (else the coarsest) starts the single-CTA solve."""
+    """Cells of the multigrid levels swept by their own launches, finest first,
+    by the library's rule on grids of even axes: a level has a coarser one
+    while every axis is at least 4; the first level of at most `coarse_cells`
+    cells (else the coarsest) starts the one-launch coarse solve."""
     dims = list(n[:dim])
     allc = []
     while True:
@@ -277,7 +277,7 @@ def mg_levels(n, dim, coarse_cells=4096):
 DENSITY_LEVELS = 1   # coarse levels rediscretised from cell densities (3D float32 path)
 
 
-def coarse_class_bytes(levels, dim, w, pre=1, post=1):
+def coarse_class_bytes(levels, dim, w, pre=1, post=1, first_colour=False):
     """Algorithmic bytes of one V-cycle, per multigrid class that spans several
     levels: the coarse tiled levels' sweeps (pre-smoothing from zero: f and
     the coefficients -> x; further sweeps x, f and the coefficients -> x), the
@@ -285,24 +285,27 @@ def coarse_class_bytes(levels, dim, w, pre=1, post=1):
     prolongations (read-add-write of the fine correction plus the coarse read),
     each level's cells times its bytes per cell. The coefficients are one
     array of cell densities on the 3D float32 path's finest level and its
-    first DENSITY_LEVELS coarse levels, else the d face arrays."""
+    first DENSITY_LEVELS coarse levels, else the d face arrays. first_colour:
+    the restriction forms the first colour's residual from its neighbours and
+    does not read f (one sweep from zero, 3D float32 path)."""
     def ncoef(i):
         return 1 if (dim == 3 and w == 4 and i <= DENSITY_LEVELS) else dim
     frac = 1.0 / 2 ** dim
     gs = sum(c * ((1 + ncoef(i) + 1) * w + (pre - 1 + post) * (1 + 1 + ncoef(i) + 1) * w)
              for i, c in enumerate(levels) if i >= 1)
-    rs = sum(c * (((2 + ncoef(i)) * w) + w * frac) for i, c in enumerate(levels))
+    xf = 1 if first_colour else 2
+    rs = sum(c * ((xf + ncoef(i)) * w + w * frac) for i, c in enumerate(levels))
     pr = sum(c * (2 * w + w * frac) for c in levels)
     return {"mg_gs_coarse_levels": gs, "mg_restrict": rs, "mg_prolong": pr}
 
 
 def step_roofline(prof, ncell, dim, w, ms_total, ms_host, peak, levels=None, vcycles=None,
-                  pre=1, post=1):
+                  pre=1, post=1, first_colour=False):
     """Compulsory bytes of the kernel classes over the whole timed region,
     divided by the headline time: the finest-grid classes (algorithmic bytes
     per cell x cells x launches) and, given the multigrid levels and the
     number of V-cycles, the classes that span the tiled levels (their bytes
-    per V-cycle x V-cycles). The single-CTA coarse solve and the once-per-solve
+    per V-cycle x V-cycles). The one-launch coarse solve and the once-per-solve
     coarsening of the coefficients are left out, so the figure is still a
     lower bound. Also the share of the host-driven step time these classes
     take."""
@@ -315,7 +318,7 @@ def step_roofline(prof, ncell, dim, w, ms_total, ms_host, peak, levels=None, vcy
             tot_ms += prof[cls][1]
             classes.append(cls)
     if levels and vcycles:
-        for cls, b in coarse_class_bytes(levels, dim, w, pre, post).items():
+        for cls, b in coarse_class_bytes(levels, dim, w, pre, post, first_colour).items():
             if cls in prof and prof[cls][0] > 0 and b > 0:
                 tot_b += b * vcycles
                 tot_ms += prof[cls][1]
@@ -645,10 +648,12 @@ def run_ours(args, rank, world, local_rank):
                              "each launch)" if args.graph else "the timed steps")}
     pre = int(p.get("mg_pre", 0) or 1)
     post = int(p.get("mg_post", 0) or 1)
-    levels = mg_levels(p["n"], p["dim"], int(p.get("mg_coarse_cells", 0) or 4096))
+    levels = mg_levels(p["n"], p["dim"], int(p.get("mg_coarse_cells", 0) or
+                                                 (40000 if p["dim"] == 3 else 4096)))
     vcycles = prof.get("mg_coarse_vcycle", (0, 0.0))[0] if "mg_coarse_vcycle" in prof else 0
     step_roof = step_roofline(prof, ncell, p["dim"], w, ms, ms_h, peak, levels=levels,
-                              vcycles=vcycles, pre=pre, post=post)
+                              vcycles=vcycles, pre=pre, post=post,
+                              first_colour=p["dim"] == 3 and w == 4 and pre == 1)
 
     # end to end through the C ABI: state from / to pinned host memory every step
     e2e = None
