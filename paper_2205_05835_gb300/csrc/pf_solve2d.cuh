@@ -621,30 +621,57 @@ PF_HD T s2_dense_part(const T* M, const T* f, int n, int t) {
     return s;
 }
 
-// Sums whose rounding is carried along: float64 sums of the float64 path,
-// (hi, lo) float pairs of the mixed one (a float64 accumulation without GB300's
-// narrow float64 pipe).
+// Sums of products as accurate as float64 ones: float64 sums of the float64
+// path; on the mixed one three floats (float64 multiply-adds would run on
+// GB300's two-lane float64 pipe). A product is split into its value and its
+// exact rounding error, the sums' rounding errors go into the second word and
+// that one's into the third. Mean error over sum |a b| of 32 random products:
+// 8e-18, float64 2e-17; with two words 1.8e-15, for 3 % less time of a 256^2
+// mixed step. The operations are spelled out, since a contracted multiply-add
+// would count an error twice.
+PF_HD float s2_add(float a, float b) {
+#ifdef __CUDA_ARCH__
+    return __fadd_rn(a, b);
+#else
+    return a + b;
+#endif
+}
+PF_HD float s2_mul(float a, float b) {
+#ifdef __CUDA_ARCH__
+    return __fmul_rn(a, b);
+#else
+    return a * b;
+#endif
+}
+PF_HD float s2_two_sum(float a, float b, float& lo) {
+    const float s = s2_add(a, b), bb = s2_add(s, -a);
+    lo = s2_add(s2_add(a, -s2_add(s, -bb)), s2_add(b, -bb));
+    return s;
+}
 struct S2AccF {
-    float s, c;
-    PF_HD void add(float v) {
-        const float t = s + v, bb = t - s;
-        c += (s - (t - bb)) + (v - bb);
-        s = t;
-    }
+    float s, c, d;
     PF_HD void add_prod(float a, float b) {
-        const float p = a * b;
-        c += fmaf(a, b, -p);
-        add(p);
+        const float p = s2_mul(a, b), e = fmaf(a, b, -p);
+        float t, v;
+        s = s2_two_sum(s, p, t);
+        const float w = s2_add(t, e);
+        c = s2_two_sum(c, w, v);
+        d = s2_add(d, s2_add(v, s2_add(s2_add(t, -w), e)));
     }
-    PF_HD void merge(float s2, float c2) {
-        add(s2);
-        c += c2;
+    // (commutative bit for bit: every CTA forms the same totals)
+    PF_HD void merge(const S2AccF& o) {
+        float t, u, v;
+        s = s2_two_sum(s, o.s, t);
+        c = s2_two_sum(c, o.c, u);
+        c = s2_two_sum(c, t, v);
+        d = s2_add(s2_add(d, o.d), s2_add(u, v));
     }
-    PF_HD double value() const { return double(s) + double(c); }
+    PF_HD double value() const { return double(s) + (double(c) + double(d)); }
 };
 struct S2AccD {
     double s;
     PF_HD void add_prod(double a, double b) { s += a * b; }
+    PF_HD void merge(const S2AccD& o) { s += o.s; }
     PF_HD double value() const { return s; }
 };
 template <typename T> struct S2AccOf { using type = S2AccD; };
