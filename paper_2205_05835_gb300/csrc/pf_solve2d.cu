@@ -43,6 +43,8 @@ struct S2Args {
     T *gx[2], *gf[2], *gw0[2], *gw1[2];   // workspace places of levels 0 and 1
     T *gdi, *gp, *gq, *ge, *gs;
     CGScalars* sc;
+    double h2;      // h^2 (mixed path: times the power of two 2^m that takes it to [1/2, 1))
+    int m;
 };
 
 // ---- totals over the cluster ----
@@ -139,8 +141,9 @@ template <typename T>
 struct S2Scal {
     T alpha, beta;
     double zq, zs, pq;
-    double ff, rr, rr0_in, eta2;
-    int done, idone, iters, it_in, outer, status, capped;
+    double ff, rr, rr0_in, rr_in, eta2;
+    int done, idone, iters, outer, status, capped, again;
+    S2Scale sca;
 };
 
 // The part of the V-cycle on the levels held by CTA 0 (the first one's right-
@@ -184,11 +187,12 @@ __device__ __forceinline__ void single_vcycle(const S2View<T>* S, int lc, int ld
 }
 
 // r = f - A x of the strip, f = sign (b - mean b), to float64 accuracy (the
-// arithmetic of k_ir_residual), stored times h^2 as the right-hand side of the
-// scaled system; per-thread ||f||^2 (first) and ||r||^2.
+// arithmetic of k_ir_residual), stored times h^2 (and its scale) as the right-hand
+// side of the scaled system; per-thread ||f||^2 (first) and ||r||^2, both times
+// their scale squared.
 template <typename T>
 __device__ __forceinline__ void s2_residual(const S2Args<T>& a, const S2View<T>& L, double mb,
-                                            bool first, T& ff, T& rr) {
+                                            bool first, const S2Scale& sca, T& ff, T& rr) {
     const int nx = L.nx;
     const bool pos = a.io.sign > 0.0;
     const int N = a.g.ncell;
@@ -199,7 +203,7 @@ __device__ __forceinline__ void s2_residual(const S2Args<T>& a, const S2View<T>&
         const float* bl = bh + N;
         const f2 mdf = df_neg(df_of(mb));
         const f2 ih2 = df_of(a.g.ih2);
-        const float h2 = float(a.g.h * a.g.h);
+        const float h2 = float(a.h2), scale = sca.scale, fscale = sca.fscale;
         s2_cells(nx, L.rows, L.lf, threadIdx.x, [&](int r, int i) {
             const int q = r * nx + i, j = L.j0 + r;
             const int idx = j * nx + i;
@@ -218,17 +222,17 @@ __device__ __forceinline__ void s2_residual(const S2Args<T>& a, const S2View<T>&
             df_face_term(w3, ch, cl, __ldcg(xh + m3), __ldcg(xl + m3), S, c);
             const f2 ax = f2_mul(two_sum(S, c), ih2);
             const f2 rv = df_add(f, df_neg(ax));
-            const float rt = __fadd_rn(rv.hi, rv.lo);
+            const float rt = __fadd_rn(rv.hi, rv.lo) * scale;
             L.f[q] = rt * h2;
             s2_start(L, i, j, q, rt * h2);
             if (first) {
-                const float ft = __fadd_rn(f.hi, f.lo);
+                const float ft = __fadd_rn(f.hi, f.lo) * fscale;
                 ff += ft * ft;
             }
             rr += rt * rt;
         });
     } else {
-        const double h2 = a.g.h * a.g.h;
+        const double h2 = a.h2;
         const double* x = a.io.x;
         s2_cells(nx, L.rows, L.lf, threadIdx.x, [&](int r, int i) {
             const int q = r * nx + i, j = L.j0 + r;
@@ -399,29 +403,39 @@ __global__ void __launch_bounds__(kS2Threads, 1) k_solve2d(const __grid_constant
     // ---- iterative refinement ----
     const double mb = a.sc->mean_b, rtol2 = a.sc->rtol2, eta2_min = a.sc->eta2_min;
     const int maxit = a.sc->maxit;
-    const double h4 = (a.g.h * a.g.h) * (a.g.h * a.g.h);
+    const double h4 = a.h2 * a.h2;
     int buf = 0;
     auto acc_of = [](T v) { A x{}; x.s = v; return x; };
     for (int outer = 0;; ++outer) {
         const bool first_res = outer == 0;
-        {
+        if (tid == 0) {
+            if (first_res) s2_scale_init(sc.sca, a.m);
+            else s2_scale_next(sc.sca, sc.rr_in);
+        }
+        __syncthreads();
+        for (int pass = 0;; ++pass) {
             T ff = T(0), rr = T(0);
-            s2_residual(a, L0, mb, first_res, ff, rr);
+            s2_residual(a, L0, mb, first_res, sc.sca, ff, rr);
             A v[2] = {acc_of(ff), acc_of(rr)}, tot{};
             cluster_totals<2>(v, tot, R, C, rank, buf);
             if (tid == 32) sc.rr = tot.value();
             __syncthreads();
             if (tid == 0) {
-                // as ir_finish
-                if (first_res) {
-                    sc.ff = tot.value();
-                    sc.iters = sc.capped = sc.done = sc.status = 0;
+                sc.rr0_in = sc.rr * h4;
+                if constexpr (std::is_same<T, float>::value) {
+                    sc.again = s2_scale_check(sc.sca, first_res, pass, rtol2, tot.value(), sc.ff,
+                                              sc.rr);
+                } else {
+                    if (first_res) sc.ff = tot.value();
+                    sc.again = 0;
                 }
+                // as ir_finish
+                if (first_res) sc.iters = sc.capped = sc.done = sc.status = 0;
                 const double rrv = sc.rr;
-                sc.rr0_in = rrv * h4;
                 sc.outer = outer + 1;
                 sc.idone = 0;
-                if (!(rrv == rrv)) {
+                if (sc.again) {
+                } else if (!(rrv == rrv)) {
                     sc.done = 1;
                     sc.status = 4;   // PF_ERR_NONFINITE
                 } else if (rrv <= rtol2 * sc.ff) {
@@ -435,6 +449,7 @@ __global__ void __launch_bounds__(kS2Threads, 1) k_solve2d(const __grid_constant
                 }
             }
             __syncthreads();
+            if (!sc.again) break;
         }
         if (sc.done || outer == 64) break;
         for (int it = 0;; ++it) {
@@ -493,6 +508,7 @@ __global__ void __launch_bounds__(kS2Threads, 1) k_solve2d(const __grid_constant
             cluster_totals<1>(rr, tot, R, C, rank, buf);
             if (tid == 0) {
                 const double v = tot.value();
+                sc.rr_in = v;
                 sc.iters += 1;
                 if (!(v == v) || v <= sc.eta2 * sc.rr0_in) {
                     sc.idone = 1;
@@ -510,7 +526,9 @@ __global__ void __launch_bounds__(kS2Threads, 1) k_solve2d(const __grid_constant
             if constexpr (sizeof(T) == sizeof(float)) {
                 float* xh = reinterpret_cast<float*>(a.io.x);
                 float* xl = xh + a.g.ncell;
-                for (int q = tid; q < n; q += kS2Threads) df_acc(xh[base + q], xl[base + q], ve[q]);
+                const float unscale = sc.sca.unscale;
+                for (int q = tid; q < n; q += kS2Threads)
+                    df_acc(xh[base + q], xl[base + q], ve[q] * unscale);
             } else {
                 for (int q = tid; q < n; q += kS2Threads) a.io.x[base + q] += ve[q];
             }
@@ -628,6 +646,13 @@ cudaError_t launch_solve2d(const S2Plan& P, const Dims& g, const Phys& ph,
     a.ge = io.e;
     a.gs = H.s2s != nullptr ? H.s2s : H.lev[0].x;
     a.sc = sc;
+    a.h2 = g.h * g.h;
+    a.m = 0;
+    if (sizeof(T) == sizeof(float)) {
+        const int e = -1 - ilogb(a.h2);
+        a.m = e < -60 ? -60 : (e > 60 ? 60 : e);
+        a.h2 = scalbn(a.h2, a.m);
+    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(P.C);
     cfg.blockDim = dim3(kS2Threads);

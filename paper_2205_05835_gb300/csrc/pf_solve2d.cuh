@@ -8,6 +8,7 @@
 #pragma once
 
 #include <math.h>
+#include <string.h>
 
 #include <type_traits>
 
@@ -676,6 +677,77 @@ struct S2AccD {
 };
 template <typename T> struct S2AccOf { using type = S2AccD; };
 template <> struct S2AccOf<float> { using type = S2AccF; };
+
+// Range of the mixed path. Its system is scaled by h^2 (times 2^m: h^2 2^m lies in
+// [1/2, 1)) and its norms are sums of float squares, so residuals are taken times
+// 2^-k, which brings their norm near 1, and the right-hand side's norm times
+// 2^-kf. Powers of two: the same bits but for what would leave float's range. k is
+// 0 in a solve's first residual, whose norm is not known, and comes from the
+// inner solve's last norm after each refinement; a norm outside [2^-16, 2^48], or
+// one that has over- or underflowed, costs further passes with the k that it asks
+// for. Right-hand sides of 1e-25 to 1e30 take the iterations of 1; without this
+// a 64^2 solve stalled below 1e-9 and a start far off left float's range.
+PF_HD double s2_pow2(int e) {   // 2^e, |e| <= 1000
+    const long long b = (long long)(1023 + e) << 52;
+    double d;
+    memcpy(&d, &b, sizeof(d));
+    return d;
+}
+PF_HD int s2_half_log2(double a) {   // exponent of the square root, a positive and normal
+    long long b;
+    memcpy(&b, &a, sizeof(b));
+    return (int)((b >> 52) - 1023) >> 1;
+}
+struct S2Scale {
+    int k, kf, m;
+    float scale, fscale;   // 2^-k, 2^-kf
+    float unscale;         // 2^(k - m): takes the inner solve's e back to x
+};
+PF_HD void s2_scale_set(S2Scale& s, int k, int kf) {
+    // (2^-k and 2^(k - m) stay normal floats)
+    k = k < s.m - 120 ? s.m - 120 : (k > s.m + 120 ? s.m + 120 : k);
+    s.k = k < -120 ? -120 : (k > 120 ? 120 : k);
+    s.kf = kf;
+    s.scale = float(s2_pow2(-s.k));
+    s.fscale = float(s2_pow2(-s.kf));
+    s.unscale = float(s2_pow2(s.k - s.m));
+}
+PF_HD void s2_scale_init(S2Scale& s, int m) {
+    s.m = m;
+    s2_scale_set(s, 0, 0);
+}
+PF_HD void s2_scale_next(S2Scale& s, double rr_in) {
+    if (rr_in > 1e-300 && rr_in < 1e300) s2_scale_set(s, s.k + s2_half_log2(rr_in), s.kf);
+}
+// After a residual pass: its squared norms ffs (first: of the right-hand side)
+// and rr as summed become ff and rr unscaled; true where the pass is to be done
+// again with the scales set here.
+PF_HD bool s2_scale_check(S2Scale& s, bool first, int pass, double rtol2, double ffs, double& ff,
+                          double& rr) {
+    constexpr int far = 64;            // one step towards a norm out of range
+    constexpr double tiny = 8e-31;     // smaller sums may have lost squares
+    const double rrs = rr;
+    int k = s.k, kf = s.kf;
+    if (first) {
+        ff = ffs * s2_pow2(2 * kf);
+        if (kf == 0) kf = !(ffs < 1e300) ? far : (ffs < tiny ? -far : 0);
+    }
+    rr = rrs * s2_pow2(2 * k);
+    const double lost = tiny * s2_pow2(2 * k);   // what rr may have lost, amply
+    if (!(rrs < 1e300)) {
+        if (pass == 0) k += far;
+    } else if (!(rr + lost <= rtol2 * ff)) {   // (else converged)
+        if (rrs < tiny) {
+            if (pass == 0) k -= far;
+        } else {
+            const int e = s2_half_log2(rrs);
+            if (e < -16 || e > 48) k += e;
+        }
+    }
+    if (pass == 2 || (k == s.k && kf == s.kf)) return false;
+    s2_scale_set(s, k, kf);
+    return true;
+}
 
 // s = A z (z: the level's x) and the products z.r, z.s and, unless first, z.q.
 template <typename T, typename A>

@@ -1,10 +1,14 @@
-"""The one-launch 2D solve: its sums of products against exact sums."""
+"""The one-launch 2D solve: its sums of products against exact sums, and the range
+of right-hand sides, box sizes and starts that it takes."""
 import ctypes
 import math
 import subprocess
 
 import numpy as np
 import pytest
+
+import pf_inputs as I
+from oracle import pf_oracle as O
 
 pytestmark = pytest.mark.gpu
 
@@ -80,3 +84,85 @@ def test_sums_of_products_are_as_accurate_as_float64_ones(pf, tmp_path, n):
         size = np.append(np.abs(prod).sum(axis=1), np.abs(prod).sum())
         count = np.append(np.full(64, n), 64 * n)
         assert (np.abs(got - want) <= 2.0 ** -53 * count * size).all()
+
+
+def beta32(phi, g, p):
+    """The mixed path's float32 face coefficients, operation by operation."""
+    f = np.float32
+    c = np.clip(phi.astype(f), f(0), f(1))
+    rho = f(p["rho_out"]) + (f(p["rho_in"]) - f(p["rho_out"])) * c
+    return [(f(1) / (f(0.5) * (rho + np.roll(rho, 1, g.axis(d))))).astype(np.float64)
+            for d in range(2)]
+
+
+def mixed_solve(pf, n, L, ratio, rhs, x0=None):
+    """(status, iterations, relative residual formed here in float64)."""
+    p = I.small_case(dim=2, n=n, precision="mixed", poisson_rtol=1e-10, L=L, R=0.25 * L,
+                     rho_in=10.0, rho_out=10.0 / ratio)
+    po = O.params_from(p)
+    g = O.Grid(2, (n, n), L)
+    phi = O.initial_phi(po).astype(np.float32).astype(np.float64)
+    sim = pf.Simulation(p, phi0=phi)
+    x, iters, rel, status = sim.poisson_solve(rhs, x0)
+    sim.close()
+    r = rhs - rhs.mean() - O.apply_poisson(beta32(phi, g, p), x, g)
+    return status, iters, np.linalg.norm(r) / np.linalg.norm(rhs - rhs.mean())
+
+
+@pytest.mark.parametrize("n", [64, 256])
+@pytest.mark.parametrize("amp", [1e-25, 1e-20, 1e-12, 1e-9, 1e6, 1e12, 1e20, 1e30])
+def test_mixed_solve_takes_any_amplitude(pf, n, amp):
+    """The solve is linear in its right-hand side, so its size changes neither the
+    convergence nor (by more than the test's own rounding) the residual. The
+    bound is rtol, plus the rounding of x as the double-float that holds it
+    (2^-46 and, in its low word, float's smallest number) through the operator."""
+    noise = I.noise((n, n), 6) - 0.5
+    st1, it1, rel1 = mixed_solve(pf, n, 1.0, 10.0, noise)
+    st, it, rel = mixed_solve(pf, n, 1.0, 10.0, amp * noise)
+    assert st1 == 0 and rel1 <= 1.1e-10
+    assert st == 0 and abs(it - it1) <= 1
+    assert rel <= 1.1e-10 + 8.0 * n * n * 2.0 ** -149 / (0.28 * amp)
+
+
+@pytest.mark.parametrize("L,amp", [(1e-6, 1.0), (1e-2, 1e-8), (1e-2, 1e8), (1e3, 1.0)])
+def test_mixed_solve_takes_any_box(pf, L, amp):
+    noise = I.noise((64, 64), 6) - 0.5
+    st1, it1, _ = mixed_solve(pf, 64, 1.0, 10.0, noise)
+    st, it, rel = mixed_solve(pf, 64, L, 10.0, amp * noise)
+    assert st1 == 0 and st == 0 and abs(it - it1) <= 1
+    assert rel <= 1.1e-10
+
+
+@pytest.mark.parametrize("ratio", [10.0, 1000.0])
+@pytest.mark.parametrize("start", [1e6, 1e13])
+def test_mixed_solve_takes_any_start(pf, ratio, start):
+    """A start whose residual is beyond float32's squares is worked off. (A constant
+    of at most its size stays in x meanwhile, and with it the rounding of a double-
+    float, 2^-47 of it times the operator's 8 max beta / h^2, so a first call may stop
+    short; x is returned with zero mean.)"""
+    rhs = I.noise((64, 64), 6) - 0.5
+    p = I.small_case(dim=2, n=64, precision="mixed", poisson_rtol=1e-10, rho_in=10.0,
+                     rho_out=10.0 / ratio)
+    sim = pf.Simulation(p)
+    x, _, rel, status = sim.poisson_solve(rhs, start * (I.noise((64, 64), 7) - 0.5))
+    floor = 2.0 ** -47 * start * 8.0 * max(0.1, 0.1 * ratio) * 64 ** 2 / 0.28
+    assert status in (pf.B.PF_OK, pf.B.PF_ERR_NOT_CONVERGED) and rel <= 1e-10 + floor
+    x, _, rel, status = sim.poisson_solve(rhs, x)
+    assert status == pf.B.PF_OK and rel <= 1e-10
+    sim.close()
+
+
+def test_mixed_solve_of_zero_and_of_a_nan(pf):
+    zero = np.zeros((64, 64))
+    p = I.small_case(dim=2, n=64, precision="mixed", poisson_rtol=1e-10)
+    sim = pf.Simulation(p)
+    x, iters, rel, status = sim.poisson_solve(zero)
+    assert status == 0 and iters == 0 and not x.any()
+    bad = I.noise((64, 64), 6)
+    bad[3, 5] = np.nan
+    with pytest.raises(pf.PFError) as e:
+        sim.poisson_solve(bad)
+    assert e.value.status == pf.B.PF_ERR_NONFINITE
+    x, iters, rel, status = sim.poisson_solve(I.noise((64, 64), 6) - 0.5)
+    assert status == 0 and rel <= 1e-10
+    sim.close()
