@@ -413,7 +413,7 @@ cudaError_t launch_solve2d(const S2Plan& P, const Dims& g, const Phys& ph,
 void launch_sum(int n, const double* x, RedBuf rb, double* out, cudaStream_t s);
 // Sets the condition of a WHILE node of a captured solve (which = 0: inner CG
 // loop, 1: outer refinement loop) from the solve's device scalars.
-void launch_set_cond(cudaGraphConditionalHandle h, const CGScalars* sc, int which, cudaStream_t s);
+void launch_set_cond(cudaGraphConditionalHandle h, CGScalars* sc, int which, cudaStream_t s);
 // The mixed path keeps the pressure and the projection's right-hand side as
 // double-floats: n float hi parts followed by n float lo parts, in the 8 n
 // bytes of a float64 array of n entries.

@@ -1222,14 +1222,19 @@ void coarse_prepare() {
 // Condition of a WHILE node of a solve captured in a CUDA graph: which = 0
 // inner CG loop (runs while the inner solve has not stopped), which = 1 outer
 // refinement loop (runs while the solve has not converged or stopped; at most
-// 64 outer residuals, as in the host-driven loop).
-__global__ void k_set_cond(cudaGraphConditionalHandle h, const CGScalars* sc, int which) {
+// 64 outer residuals, as in the host-driven loop). A solve that stops there
+// latches its status: the step's later solves overwrite done.
+__global__ void k_set_cond(cudaGraphConditionalHandle h, CGScalars* sc, int which) {
     unsigned v;
-    if (which == 0) v = (sc->done || sc->idone) ? 0u : 1u;
-    else v = (!sc->done && sc->outer < 64) ? 1u : 0u;
+    if (which == 0) {
+        v = (sc->done || sc->idone) ? 0u : 1u;
+    } else {
+        v = (!sc->done && sc->outer < 64) ? 1u : 0u;
+        if (!sc->done && v == 0u && sc->status == 0) sc->status = 3;   // PF_ERR_NOT_CONVERGED
+    }
     cudaGraphSetConditional(h, v);
 }
-void launch_set_cond(cudaGraphConditionalHandle h, const CGScalars* sc, int which, cudaStream_t s) {
+void launch_set_cond(cudaGraphConditionalHandle h, CGScalars* sc, int which, cudaStream_t s) {
     k_set_cond<<<1, 1, 0, s>>>(h, sc, which);
 }
 

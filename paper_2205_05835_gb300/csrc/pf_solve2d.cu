@@ -544,7 +544,9 @@ __global__ void __launch_bounds__(kS2Threads, 1) k_solve2d(const __grid_constant
         o->done = sc.done;
         o->idone = 1;
         o->capped = sc.capped;
-        if (o->status == 0) o->status = sc.status;
+        // (latched: in a graph the step's later solves overwrite done)
+        const int status = sc.done ? sc.status : 3;   // PF_ERR_NOT_CONVERGED: 64 refinements
+        if (o->status == 0) o->status = status;
     }
     cluster_sync(C);   // no CTA leaves while another may read its memory
 }

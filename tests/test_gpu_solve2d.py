@@ -166,3 +166,41 @@ def test_mixed_solve_of_zero_and_of_a_nan(pf):
     x, iters, rel, status = sim.poisson_solve(I.noise((64, 64), 6) - 0.5)
     assert status == 0 and rel <= 1e-10
     sim.close()
+
+
+# tolerances between the residuals at which rounding stops the two solves (64
+# refinements): measured 9.6e-12 and at most 3.1e-12 at 256^2, 6.2e-11 and at most 3.1e-12 at
+# 640^2 (beyond the one-launch solve), 5.3e-13 and at most 8.2e-14 at 64^3
+@pytest.mark.parametrize("n,rtol", [((256, 256), 6e-12), ((640, 640), 2e-11),
+                                    ((64, 64, 64), 2e-13)])
+def test_graph_reports_a_solve_that_stops_at_the_refinement_limit(pf, n, rtol):
+    """Two forward-Euler steps of one call in graph mode, at density ratio 1 from a
+    smooth potential flow. The first solve's pressure is large against its right-
+    hand side, so its rounding keeps it above rtol; the second's right-hand side
+    is what the projection left, which is rough, and converges. The first one's
+    failure is reported."""
+    p = I.small_case(dim=len(n), n=n[0], precision="mixed", poisson_rtol=rtol, rho_in=1.0,
+                     rho_out=1.0, sigma=0.0, mu_in=0.0, mu_out=0.0, scheme="fe",
+                     poisson_maxit=5000, use_graph=1, pert_mode=0, pert_amp=0.0)
+    t = 2.0 * np.pi * np.arange(n[0]) / n[0]
+    tc = t + np.pi / n[0]
+    u = (1.0 + 0.5 * np.cos(tc + 1.1))[:, None] * np.sin(t + 0.3)[None, :]
+    v = 0.5 * np.sin(t + 1.1)[:, None] * np.cos(tc + 0.3)[None, :]
+
+    def fresh():
+        sim = pf.Simulation(p)
+        sim.set_field("u", np.broadcast_to(u, sim.shape))
+        sim.set_field("v", np.broadcast_to(v, sim.shape))
+        return sim
+
+    sim = fresh()
+    with pytest.raises(pf.PFError) as e:
+        sim.step(1)
+    assert e.value.status == pf.B.PF_ERR_NOT_CONVERGED
+    sim.step(1)   # the second step's solve converges, and the latch is clear
+    sim.close()
+    sim = fresh()
+    with pytest.raises(pf.PFError) as e:
+        sim.step(2)
+    assert e.value.status == pf.B.PF_ERR_NOT_CONVERGED
+    sim.close()
