@@ -309,46 +309,10 @@ struct ImplT final : Impl {
         build_levels(false);
     }
 
-    // Geometry of the multigrid hierarchy: every axis of 2 cells or more is
-    // halved (an odd one to floor(n / 2), its last coarse cell taking three
-    // children; one cell along an axis couples to nothing there), until every
-    // axis has at most 3 cells. Any size reaches a bottom level that a few
-    // sweeps solve; a hierarchy that stops at the first odd or short axis needs
-    // 4 n^2 sweeps of an n-cell axis there (a 160 x 120 x 72 step spent 135 of
-    // its 143 ms in the 20 x 15 x 9 bottom level, 200 x 136 262 of 266 ms in
-    // 25 x 17). Keeping a short axis uncoarsened instead of taking it to one
-    // cell leaves its coupling dominant and point sweeps stall (7 x 63 to 1e-9: 72
-    // iterations, against fewer than 34).
-    // even_only: halvings of even axes alone (the smaller workspace of
-    // pf_poisson_solve_static at its capacity limit).
+    // even_only: see mg_geometry (the smaller workspace of pf_poisson_solve_static
+    // at its capacity limit)
     void build_levels(bool even_only) {
-        H.nlev = 1;
-        H.lev[0].g = g;
-        for (int d = 0; d < 3; ++d) H.lev[0].lastw[d] = 1.f;
-        for (;;) {
-            MGLevel<T>& F = H.lev[H.nlev - 1];
-            const int n[3] = {F.g.nx, F.g.ny, F.g.nz};
-            int m[3] = {n[0], n[1], n[2]};
-            bool any = false, all_even = true;
-            for (int d = 0; d < 3; ++d) {
-                F.cf[d] = 1;
-                if (d >= DIM) continue;
-                if (n[d] < 4 || n[d] % 2 != 0) all_even = false;
-                if (n[d] >= 4) any = true;
-                if (n[d] >= 2) {
-                    F.cf[d] = 2;
-                    m[d] = n[d] / 2;
-                }
-            }
-            if (H.nlev == kMaxLevels || !any || (even_only && !all_even)) break;
-            MGLevel<T>& C = H.lev[H.nlev];
-            C.g = make_dims(m[0], m[1], m[2], F.g.h * 2.0);
-            C.g.wall_y = F.g.wall_y;
-            for (int d = 0; d < 3; ++d)
-                C.lastw[d] = F.cf[d] == 1 ? F.lastw[d]
-                                          : 0.5f * (F.lastw[d] + (n[d] % 2 ? 2.f : 1.f));
-            ++H.nlev;
-        }
+        mg_geometry(H, g, DIM, even_only);
         for (int l = 0; l < kMaxLevels; ++l) H.lev[l].x2 = nullptr;
         H.first_coarse = H.nlev - 1;
         const int coarse_cells = prm.mg_coarse_cells > 0 ? prm.mg_coarse_cells : 4096;
@@ -488,9 +452,12 @@ struct ImplT final : Impl {
         }
         H.s2s = DIM == 2 ? cv.take<T>(n) : nullptr;
         // inverse diagonals of the float64 levels outside the coarse kernel (2D:
-        // grids beyond the one-launch solve)
+        // grids that do not take the one-launch solve)
         for (int l = 0; l < kMaxLevels; ++l) H.lev[l].di = nullptr;
-        if (sizeof(T) == sizeof(double) && (DIM == 3 || n > (size_t)kSolve2dCells))
+        S2Plan one;
+        if (sizeof(T) == sizeof(double) &&
+            (DIM == 3 || !s2_plan<T>(H, s2_limits<T>(kS2MaxCTAs, s2_dynamic_smem<T>()), true, true,
+                                     one)))
             for (int l = 0; l < H.first_coarse; ++l) H.lev[l].di = cv.take<T>(H.lev[l].g.ncell);
         // second buffers for the one-pass out-of-place sweeps (3D float32 levels
         // below the single-CTA levels)

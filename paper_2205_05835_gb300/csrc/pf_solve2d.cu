@@ -30,7 +30,6 @@ namespace pf {
 namespace {
 
 constexpr int kS2Warps = kS2Threads / 32;
-constexpr size_t kS2SmemMax = 227 * 1024;   // shared memory of a CTA
 
 template <typename T>
 struct S2Args {
@@ -551,37 +550,12 @@ __global__ void __launch_bounds__(kS2Threads, 1) k_solve2d(const __grid_constant
     cluster_sync(C);   // no CTA leaves while another may read its memory
 }
 
-// Largest strip (cells of level 0 per CTA) the cluster takes. Beyond it the
-// kernels on the whole chip are faster: a mixed step of 512^2 takes 3.7 ms
-// here and 4.5 ms there, of 576^2 7.6 and 4.7 ms; a float64 one of 512^2 10.2
-// and 11.0 ms (larger ones do not fit).
-constexpr int kMaxCtaCells = kSolve2dCells / kS2MaxCTAs;
-
 // dynamic shared memory left beside the kernel's static arrays
 template <typename T>
 size_t dynamic_smem() {
     cudaFuncAttributes at;
     if (cudaFuncGetAttributes(&at, k_solve2d<T>) != cudaSuccess) return 0;
     return kS2SmemMax - ((at.sharedSizeBytes + 1023) & ~(size_t)1023);
-}
-
-template <typename T>
-S2Limits limits(int max_cluster) {
-    // Cycles measured at 64^2 .. 256^2: a phase of a cluster costs about 900
-    // beside its cells, one of a CTA 400. The fused interpolation has 31 instructions a cell instead of 4, too many for
-    // the float64 pipe.
-    const bool f32 = sizeof(T) == 4;
-    S2Limits m;
-    m.max_cluster = max_cluster;
-    m.dense_cells = f32 ? kS2DenseMax : 16;
-    m.fused_cells = f32 ? 2048 : 0;
-    m.cta_cells = kMaxCtaCells;
-    m.cell = f32 ? 8.f : 28.f;
-    m.single_cell = f32 ? 5.f : 13.f;
-    m.phase = 900.f;
-    m.cta_phase = 400.f;
-    m.smem_bytes = dynamic_smem<T>();
-    return m;
 }
 
 template <typename T>
@@ -622,7 +596,8 @@ void solve2d_prepare() {
 template <typename T>
 bool solve2d_plan(const MGHier<T>& H, bool beta_global, S2Plan& P) {
     const int mc = max_cluster<T>();
-    return mc > 0 && s2_plan<T>(H, limits<T>(mc), beta_global, H.s2s != nullptr, P);
+    return mc > 0 && s2_plan<T>(H, s2_limits<T>(mc, dynamic_smem<T>()), beta_global,
+                                H.s2s != nullptr, P);
 }
 
 template <typename T>

@@ -70,61 +70,68 @@ inline int s2_max_rows(const S2Plan& P, int l) {
 
 // What decides the plan: the largest cluster, the dense level's cells, the
 // strip's cells up to which the interpolation joins the first post class, the
-// dynamic shared memory, and a cost model of an iteration in cycles: per cell
-// of the largest strip, per cell of the levels of CTA 0, per phase of a cluster
-// and of a CTA.
+// largest strip (cells of level 0 per CTA), that of a split that is not the
+// cheapest, the dynamic shared memory, and a cost model of an iteration in
+// cycles: per cell of the largest strip, per cell of the levels of CTA 0, per
+// phase of a cluster and of a CTA.
 struct S2Limits {
-    int max_cluster, dense_cells, fused_cells, cta_cells;
+    int max_cluster, dense_cells, fused_cells, cta_cells, other_cells;
     float cell, single_cell, phase, cta_phase;
     size_t smem_bytes;
 };
-
-// Fits the solve of a hierarchy into a cluster's shared memory: false when it
-// does not (too large a grid: more than cta_cells cells a CTA). beta_global:
-// the face coefficients also exist in the workspace; s_global: so does a place
-// for s.
+constexpr int kS2DenseMax = 32;   // cells of a dense level (see s2_gj_publish)
+// Largest strip. Beyond it the kernels on the whole chip are faster: a mixed step
+// of 512^2 takes 3.7 ms in the cluster and 4.5 ms there, of 576^2 7.6 and 4.7 ms; a
+// float64 one of 512^2 10.2 and 11.0 ms (larger ones do not fit).
+constexpr int kS2CtaCells = kSolve2dCells / kS2MaxCTAs;
+// Shared memory of a CTA, and what the kernel's static arrays leave of it (the
+// launch asks the kernel itself; this decides the workspace, without a GPU).
+constexpr size_t kS2SmemMax = 227 * 1024;
 template <typename T>
-inline bool s2_plan(const MGHier<T>& H, const S2Limits& lim, bool beta_global, bool s_global,
-                    S2Plan& P) {
-    if (H.nlev < 2 || H.lev[0].g.nz != 1) return false;
-    P.pre = H.pre;
-    P.post = H.post;
-    for (int l = 0; l < H.nlev; ++l) {
-        S2Lev& L = P.lev[l];
-        L.nx = H.lev[l].g.nx;
-        L.ny = H.lev[l].g.ny;
-        L.cfx = H.lev[l].cf[0];
-        L.cfy = H.lev[l].cf[1];
-        L.qx = H.lev[l].lastw[0];
-        L.qy = H.lev[l].lastw[1];
-    }
+constexpr size_t s2_dynamic_smem() {
+    return kS2SmemMax - (sizeof(T) == 4 ? 5 : 17) * 1024;
+}
+
+template <typename T>
+inline S2Limits s2_limits(int max_cluster, size_t smem_bytes) {
+    // Cycles measured at 64^2 .. 256^2: a phase of a cluster costs about 900
+    // beside its cells, one of a CTA 400. The fused interpolation has 31
+    // instructions a cell instead of 4, too many for the float64 pipe.
+    const bool f32 = sizeof(T) == 4;
+    S2Limits m;
+    m.max_cluster = max_cluster;
+    m.dense_cells = f32 ? kS2DenseMax : 16;
+    m.fused_cells = f32 ? 2048 : 0;
+    m.cta_cells = kS2CtaCells;
+    m.other_cells = f32 ? 13500 : 9500;
+    m.cell = f32 ? 8.f : 28.f;
+    m.single_cell = f32 ? 5.f : 13.f;
+    m.phase = 900.f;
+    m.cta_phase = 400.f;
+    m.smem_bytes = smem_bytes;
+    return m;
+}
+
+// Modelled cycles of an iteration of a split (C and lc chosen).
+inline float s2_cost(const S2Plan& P, int nlev, const S2Limits& lim) {
     auto cells = [&](int l) { return P.lev[l].nx * P.lev[l].ny; };
-    // the bottom must be small (a hierarchy of even halvings alone may not be)
-    if (cells(H.nlev - 1) > lim.dense_cells) return false;
-    // the split with the least modelled cost: more cluster levels make the
-    // strips coarser (unequal), fewer leave more to CTA 0
-    float best = -1.f;
-    S2Plan Q = P;
-    for (int lc = 1; lc < H.nlev && lc < kS2MaxCluster; ++lc)
-        for (int C = 1; C <= lim.max_cluster && C <= kS2MaxCTAs && C <= P.lev[lc].ny; C *= 2) {
-            Q.lc = lc;
-            Q.C = C;
-            float c = 5.f * float(lc) * (C == 1 ? lim.cta_phase : lim.phase);
-            for (int l = 0; l < lc; ++l)
-                c += (l == 0 ? lim.cell : lim.single_cell) * float(s2_max_rows(Q, l) * P.lev[l].nx);
-            for (int l = lc; l < H.nlev && cells(l) > lim.dense_cells; ++l)
-                c += lim.single_cell * float(cells(l)) + 5.f * lim.cta_phase;
-            if (best < 0.f || c < best) {
-                best = c;
-                P.lc = lc;
-                P.C = C;
-            }
-        }
-    if (s2_max_rows(P, 0) * P.lev[0].nx > lim.cta_cells) return false;
+    float c = 5.f * float(P.lc) * (P.C == 1 ? lim.cta_phase : lim.phase);
+    for (int l = 0; l < P.lc; ++l)
+        c += (l == 0 ? lim.cell : lim.single_cell) * float(s2_max_rows(P, l) * P.lev[l].nx);
+    for (int l = P.lc; l < nlev && cells(l) > lim.dense_cells; ++l)
+        c += lim.single_cell * float(cells(l)) + 5.f * lim.cta_phase;
+    return c;
+}
+
+// Places a plan's arrays (C and lc chosen): false when they do not fit.
+inline bool s2_place(S2Plan& P, const S2Limits& lim, size_t elem, bool beta_global,
+                     bool s_global) {
+    auto cells = [&](int l) { return P.lev[l].nx * P.lev[l].ny; };
+    if ((long long)s2_max_rows(P, 0) * P.lev[0].nx > lim.cta_cells) return false;
     P.ld = P.lc;
     while (cells(P.ld) > lim.dense_cells) ++P.ld;
     long long off = 0;
-    const long long cap = (long long)(lim.smem_bytes / sizeof(T));
+    const long long cap = (long long)(lim.smem_bytes / elem);
     auto fits = [&](int* slot, long long n) {
         *slot = -1;
         if (off + n + 3 > cap) return false;
@@ -149,6 +156,7 @@ inline bool s2_plan(const MGHier<T>& H, const S2Limits& lim, bool beta_global, b
     int* slots[9] = {&L.ox, &L.ow0, &L.ow1, &L.of, &L.od, &P.os, &P.oq, &P.op, &P.oe};
     for (int s = 0; s < 9; ++s) fits(slots[s], n0);
     if (P.os < 0 && !s_global && L.ox < 0) return false;   // (x's workspace place is free)
+    if (!beta_global && (L.ow0 < 0 || L.ow1 < 0)) return false;
     P.fused = 0;
     for (int l = 0; l < P.ld; ++l) {
         const S2Lev &F = P.lev[l], &N = P.lev[l + 1];
@@ -156,9 +164,56 @@ inline bool s2_plan(const MGHier<T>& H, const S2Limits& lim, bool beta_global, b
         if (even && N.qx == 1.f && N.qy == 1.f && s2_max_rows(P, l) * F.nx <= lim.fused_cells)
             P.fused |= 1u << l;
     }
-    if (!beta_global && (L.ow0 < 0 || L.ow1 < 0)) return false;
     P.elems = (int)off;
     return true;
+}
+
+// The plan of a hierarchy's solve: of the splits that fit a cluster's shared
+// memory the one with the least modelled cost (more cluster levels make the
+// strips coarser and unequal, fewer leave more to CTA 0); false when none does.
+// beta_global: the face coefficients also exist in the workspace; s_global: so
+// does a place for s.
+template <typename T>
+inline bool s2_plan(const MGHier<T>& H, const S2Limits& lim, bool beta_global, bool s_global,
+                    S2Plan& P) {
+    if (H.nlev < 2 || H.lev[0].g.nz != 1) return false;
+    S2Plan Q;
+    Q.pre = H.pre;
+    Q.post = H.post;
+    for (int l = 0; l < H.nlev; ++l) {
+        S2Lev& L = Q.lev[l];
+        L.nx = H.lev[l].g.nx;
+        L.ny = H.lev[l].g.ny;
+        L.cfx = H.lev[l].cf[0];
+        L.cfy = H.lev[l].cf[1];
+        L.qx = H.lev[l].lastw[0];
+        L.qy = H.lev[l].lastw[1];
+    }
+    // the bottom must be small (a hierarchy of even halvings alone may not be)
+    if (H.lev[H.nlev - 1].g.ncell > lim.dense_cells) return false;
+    float best = -1.f, least = -1.f;
+    for (int lc = 1; lc < H.nlev && lc < kS2MaxCluster; ++lc)
+        for (int C = 1; C <= lim.max_cluster && C <= kS2MaxCTAs && C <= Q.lev[lc].ny; C *= 2) {
+            Q.lc = lc;
+            Q.C = C;
+            const float c = s2_cost(Q, H.nlev, lim);
+            if (least < 0.f || c < least) least = c;
+            if (best >= 0.f && c >= best) continue;
+            if (!s2_place(Q, lim, sizeof(T), beta_global, s_global)) continue;
+            best = c;
+            P = Q;
+        }
+    if (best < 0.f) return false;
+    // A split that is not the cheapest has unequal strips or more in CTA 0, and
+    // the kernels overtake it sooner, on odd sizes (three classes a sweep) sooner
+    // yet. Graph steps, strip's cells: cluster and kernels. Float64: 268^2 (7504)
+    // 5.0 and 6.3 ms, 468 x 156 (9360) 6.3 and 7.6, 692 x 144 (11072) 7.0 and 6.7, 548 x 164
+    // (10960) 7.8 and 6.3; odd: 313 x 54 (3130) 5.5 and 8.5, 301 x 299 (8428) 13.1 and
+    // 9.5. Mixed: 468 x 276 (13104) 2.7 and 3.0, 704 x 188 (14080) equal, 580 x 276
+    // (16240) 4.8 and 3.3.
+    const int n0 = s2_max_rows(P, 0) * P.lev[0].nx;
+    const bool odd = (P.lev[0].nx | P.lev[0].ny) & 1;
+    return best == least || n0 <= (odd ? lim.other_cells / 2 : lim.other_cells);
 }
 
 // One level as a CTA sees it: its rows [j0, j0 + rows) (pointers at row j0),
@@ -540,7 +595,6 @@ PF_HD void s2_dense_fill(const S2View<T>& L, T* M, int t) {
 // reciprocal of the current matrix into one of two buffers, step reads them.
 // One barrier a step. (64 cells took 45 us a solve, more than the level that
 // 16 to 27 cells add costs in ten V-cycles.)
-constexpr int kS2DenseMax = 32;                       // cells of a dense level
 constexpr int kS2Col = kS2DenseMax, kS2ColRow = 2 * kS2DenseMax + 1;   // the row's offset; size
 template <typename T>
 PF_HD void s2_gj_publish(const T (&m)[2], int n, int k, T* buf, int t) {

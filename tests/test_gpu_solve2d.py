@@ -204,3 +204,36 @@ def test_graph_reports_a_solve_that_stops_at_the_refinement_limit(pf, n, rtol):
         sim.step(2)
     assert e.value.status == pf.B.PF_ERR_NOT_CONVERGED
     sim.close()
+
+
+# the last three: the next split's strip is too large, or none fits
+@pytest.mark.parametrize("n,precision,cluster",
+                         [((64, 64), "fp64", True), ((512, 512), "fp64", True),
+                          ((268, 268), "fp64", True), ((512, 40), "fp64", True),
+                          ((300, 300), "fp64", True), ((468, 156), "fp64", True),
+                          ((313, 54), "fp64", True), ((468, 276), "mixed", True),
+                          ((512, 512), "mixed", True), ((548, 164), "fp64", False),
+                          ((580, 276), "mixed", False), ((1000, 200), "fp64", False)])
+def test_which_solve_a_grid_takes(pf, n, precision, cluster):
+    rtol = 1e-11 if precision == "fp64" else 1e-10
+    p = I.small_case(dim=2, n=n[0], precision=precision, poisson_rtol=rtol,
+                     R=0.25 * min(1.0, n[1] / n[0]))
+    p["n"] = n + (1,)
+    po = O.params_from(p)
+    g = O.Grid(2, n, p["L"])
+    phi = O.initial_phi(po).astype(np.float32).astype(np.float64)
+    rhs = I.noise(g.shape, 6) - 0.5
+    rhs -= rhs.mean()
+    sim = pf.Simulation(p, phi0=phi)
+    x, iters, rel, status = sim.poisson_solve(rhs)
+    ran = pf.pf_profile_read(sim.ctx)
+    sim.close()
+    assert (ran.get("solve2d_cluster", (0, 0.0))[0] > 0) == cluster
+    assert (ran.get("cg_update", (0, 0.0))[0] > 0) != cluster
+    beta = O.face_beta(phi, g, po) if precision == "fp64" else beta32(phi, g, p)
+    r = rhs - O.apply_poisson(beta, x, g)
+    # rounding of x (2^-47 for a double-float, 2^-52 for float64) through the operator
+    eps = 2.0 ** -47 if precision == "mixed" else 2.0 ** -52
+    floor = 8.0 * eps * max(b.max() for b in beta) / g.h ** 2 * np.linalg.norm(x)
+    assert status == 0 and iters <= 40
+    assert np.linalg.norm(r) <= 1.01 * rtol * np.linalg.norm(rhs) + floor
