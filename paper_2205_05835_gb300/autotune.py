@@ -46,17 +46,22 @@ MARGIN = 0.01                            # relative gain needed to leave a defau
 INNER_TOLS = (1e-6, 1e-5, 1e-4, 1e-3)   # the first is the library's default
 SWEEP_TILES = (0, 1, 2, 3, 4)           # the first is the library's default
 
+# Part of every cache key: raised whenever the candidates or what the library makes
+# of them change, so that a stored choice is not used for something else (1:
+# mg_coarse_cells 4096 was the default, 2: 0, the library's rule)
+SETTINGS_VERSION = 2
+
 _cache: dict = {}
 
 
 def signature(p: dict, tune_inner: bool = False) -> str:
-    """What the best launch shape depends on: the grid, precision, model,
+    """What the best launch shape depends on: the version of the settings, the grid, precision, model,
     force, density ratio, walls, execution mode, the solve's tolerances (a
     tight poisson_rtol favours stronger V-cycles; a preset inner_tol is part of
     the problem) and whether the inner tolerance was tuned as well."""
     n = tuple(int(v) for v in p["n"])
     ratio = round(float(p["rho_in"]) / float(p["rho_out"]), 6)
-    return json.dumps([int(p["dim"]), n, str(p.get("precision")), str(p.get("model")),
+    return json.dumps([f"v{SETTINGS_VERSION}", int(p["dim"]), n, str(p.get("precision")), str(p.get("model")),
                        str(p.get("force")), ratio, int(p.get("wall_y", 0) or 0),
                        int(p.get("use_graph", 0) or 0), float(p.get("poisson_rtol", 0.0) or 0.0),
                        float(p.get("inner_tol", 0.0) or 0.0), bool(tune_inner)])
