@@ -23,7 +23,8 @@ converged answer (every candidate solves to the same poisson_rtol):
 
 Each candidate gets a fresh context on the same parameters, runs `warm`
 steps, then `steps` timed steps (pf_step synchronises, so the host clock
-brackets device work); the fastest candidate wins, except that the library's
+brackets device work; candidates that are one and the same on a 2D grid solved
+in one launch are timed once); the fastest candidate wins, except that the library's
 defaults are kept unless a candidate beats them by more than MARGIN (a few
 timed steps do not resolve smaller differences). Results are cached per
 signature in memory and, given a path, in a JSON file, so a batch of many
@@ -78,6 +79,17 @@ def _time_candidate(pf, p: dict, cand: dict, steps: int, warm: int) -> float:
         sim.close()
 
 
+def _one_launch(pf, p: dict) -> bool:
+    """Whether the 2D grid's solves run in one launch, where mg_coarse_cells has no
+    effect."""
+    sim = pf.Simulation(dict(p))
+    try:
+        sim.step(1)
+        return pf.pf_profile_read(sim.ctx).get("solve2d_cluster", (0, 0.0))[0] > 0
+    finally:
+        sim.close()
+
+
 def tune(p: dict, candidates=CANDIDATES, steps: int = 2, warm: int = 1,
          cache_path: str | None = None, tune_inner: bool = False) -> dict:
     """Best candidate for the parameters p: {"choice": {...}, "ms_per_step":
@@ -90,10 +102,20 @@ def tune(p: dict, candidates=CANDIDATES, steps: int = 2, warm: int = 1,
             _cache.update(json.load(f))
     if key in _cache:
         return dict(_cache[key], cached=True)
-    times = {}
+    times, same, one_launch = {}, {}, None
     for c in candidates:
-        times[json.dumps(c, sort_keys=True)] = 1e3 * _time_candidate(pf, p, c, steps, warm)
-    best = min(times, key=times.get)
+        k = json.dumps(c, sort_keys=True)
+        first = same.setdefault(json.dumps(dict(c, mg_coarse_cells=0), sort_keys=True), k)
+        if first != k and int(p["dim"]) == 2:
+            # differs in mg_coarse_cells alone
+            if one_launch is None:
+                one_launch = _one_launch(pf, p)
+            if one_launch:
+                times[k] = times[first]
+                continue
+        times[k] = 1e3 * _time_candidate(pf, p, c, steps, warm)
+    # of equal ones the library's own rule
+    best = min(times, key=lambda k: (times[k], json.loads(k).get("mg_coarse_cells", 0) != 0))
     dkey = json.dumps(DEFAULT_SHAPE, sort_keys=True)
     if dkey in times and times[dkey] <= times[best] * (1.0 + MARGIN):
         best = dkey

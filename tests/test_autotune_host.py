@@ -36,3 +36,23 @@ def test_a_cache_of_other_settings_is_not_used(autotune, monkeypatch, tmp_path):
     assert again["cached"] and again["choice"] == r["choice"]
     assert len(timed) == len(autotune.CANDIDATES)
     autotune._cache.clear()
+
+
+@pytest.mark.parametrize("one", [True, False])
+def test_candidates_that_are_the_same_are_timed_once(autotune, monkeypatch, one):
+    """On a 2D grid solved in one launch mg_coarse_cells does nothing: one timing for
+    each pair of sweep counts, and the library's rule among equals."""
+    timed = []
+
+    def fake(pf, p, c, steps, warm):
+        timed.append(c)
+        return 0.5 if c["mg_pre"] == 2 else 1.0
+    monkeypatch.setattr(autotune, "_time_candidate", fake)
+    monkeypatch.setattr(autotune, "_one_launch", lambda pf, p: one, raising=False)
+    autotune._cache.clear()
+    r = autotune.tune(dict(P, dim=2, n=(64, 64, 1)))
+    sweeps = {(c["mg_pre"], c["mg_post"]) for c in autotune.CANDIDATES}
+    assert len(timed) == (len(sweeps) if one else len(autotune.CANDIDATES))
+    assert len(r["ms_per_step"]) == len(autotune.CANDIDATES)
+    assert r["choice"] == {"mg_coarse_cells": 0, "mg_pre": 2, "mg_post": 2}
+    autotune._cache.clear()
