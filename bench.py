@@ -245,6 +245,10 @@ def algo_bytes_per_cell(cls, dim, w, fused_stage=False):
         # x += e with x a double-float (float64 path: float64) pressure
         "ir_addcorr": 2 * (8 if w == 4 else w) + w,
         "gamma": d * w,
+        # a whole 2D solve in one launch: read phi, b and x (float64 or double-float);
+        # write x and the d face arrays. What bounds it is its chain of phases, so
+        # the fraction is small
+        "solve2d_cluster": w + 3 * 8 + d * w,
     }
     return table.get(cls)
 
@@ -252,7 +256,8 @@ def algo_bytes_per_cell(cls, dim, w, fused_stage=False):
 # kernel classes that work on the finest grid (one launch covers every cell);
 # the coarse multigrid classes run on levels of 1/2^d, 1/4^d, ... the cells
 FINEST_CLASSES = ("mg_gs_level0", "cg_dir_spmv", "cg_update", "ir_residual_f64", "stage",
-                  "cell_pass", "correct", "divergence", "beta0_f64", "ir_addcorr", "gamma")
+                  "cell_pass", "correct", "divergence", "beta0_f64", "ir_addcorr", "gamma",
+                  "solve2d_cluster")
 
 
 def mg_levels(n, dim, coarse_cells=4096):

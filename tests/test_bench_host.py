@@ -65,3 +65,14 @@ def test_multilevel_classes_in_the_step_roofline(bench):
     r1 = bench.step_roofline(prof, lv[0], 3, 4, 4.0, 8.0, 100.0, levels=lv, vcycles=10)
     assert r1["bytes"] == r0["bytes"] + 10 * sum(cb.values())
     assert "mg_prolong" in r1["classes"] and "mg_coarse_vcycle" not in r1["classes"]
+
+
+def test_the_one_launch_2d_solve_counts_in_the_step_roofline(bench):
+    """A 2D step is stage kernels and four one-launch solves: each solve reads phi, b
+    and x and writes x and two face arrays (36 B a cell mixed, 48 float64)."""
+    assert bench.algo_bytes_per_cell("solve2d_cluster", 2, 4) == 36
+    assert bench.algo_bytes_per_cell("solve2d_cluster", 2, 8) == 48
+    prof = {"stage": (4, 1.0), "cell_pass": (4, 0.5), "solve2d_cluster": (4, 6.0)}
+    r = bench.step_roofline(prof, 1000, 2, 4, ms_total=8.0, ms_host=8.0, peak=100.0)
+    assert "solve2d_cluster" in r["classes"]
+    assert r["their_time_share"] == pytest.approx(7.5 / 8.0)
