@@ -51,7 +51,8 @@ typedef enum {
     PF_OK = 0,
     PF_ERR_INVALID = 1,        /* bad parameter, size or pointer */
     PF_ERR_CUDA = 2,           /* a CUDA runtime call failed; see pf_last_error */
-    PF_ERR_NOT_CONVERGED = 3,  /* Poisson solve hit poisson_maxit before poisson_rtol */
+    PF_ERR_NOT_CONVERGED = 3,  /* Poisson solve hit poisson_maxit, or 64 refinements, before
+                                  poisson_rtol */
     PF_ERR_NONFINITE = 4,      /* NaN or Inf found in the state */
     PF_ERR_UNBOUNDED = 5,      /* phi left [-bound_tol, 1 + bound_tol] (when checked) */
     PF_ERR_TIMEOUT = 6,        /* a bounded device wait gave up (TMA-staged sweeps) */
@@ -249,7 +250,8 @@ int pf_profile_read(pf_ctx* ctx, pf_profile_entry* out, int max_entries, int res
  * phi, rhs: float64 device arrays of nx*ny*nz (inputs); x: float64 device
  * array, initial guess on entry and solution on exit. stream: cudaStream_t as
  * void*. Synchronises the stream before returning. iters, relres: optional.
- * Returns PF_ERR_NOT_CONVERGED (x still written) when poisson_maxit is hit.
+ * Returns PF_ERR_NOT_CONVERGED (x still written) when poisson_maxit, or the limit of 64
+ * refinements, is hit.
  * The first call on a device looks up the array's device address (with that
  * device current), so make it before any stream capture. The array keeps the
  * last call's contents and every call clears what must start at zero; calls

@@ -820,7 +820,8 @@ struct ImplT final : Impl {
             // completion counter is cleared for the next solve
             if (stt == PF_ERR_TIMEOUT)
                 CK(cudaMemsetAsync(rb.counter, 0, 4 * sizeof(unsigned int), st));
-            err = stt == PF_ERR_NOT_CONVERGED ? "Poisson solve reached poisson_maxit"
+            err = stt == PF_ERR_NOT_CONVERGED
+                      ? "Poisson solve reached poisson_maxit or 64 refinements"
                   : stt == PF_ERR_TIMEOUT
                       ? "a bounded wait of the TMA-staged sweep gave up (copies did not land)"
                       : "non-finite value in the Poisson solve";

@@ -12,7 +12,7 @@
 // partial sums in the same order.
 //
 // Measured: four 64^2 float64 steps 27.6 -> 4.2 ms, four mixed 256^2 steps at
-// density ratio 1000 (54 iterations a step) 21.4 -> 7.6 ms, two 128^2 float64
+// density ratio 1000 (54 iterations a step) 21.4 -> 7.8 ms, two 128^2 float64
 // steps between walls 26.1 -> 4.0 ms. What bounds it is the chain: some 35
 // barriers an iteration (588 cycles across the cluster, 44 in a CTA), each with
 // one or two cells a thread in between (some 450 cycles of issue and latency);

@@ -80,9 +80,10 @@ struct S2Limits {
     size_t smem_bytes;
 };
 constexpr int kS2DenseMax = 32;   // cells of a dense level (see s2_gj_publish)
-// Largest strip. Beyond it the kernels on the whole chip are faster: a mixed step
-// of 512^2 takes 3.7 ms in the cluster and 4.5 ms there, of 576^2 7.6 and 4.7 ms; a
-// float64 one of 512^2 10.2 and 11.0 ms (larger ones do not fit).
+// Largest strip. Beyond it the kernels on the whole chip are faster: a graph step
+// of a 512^2 drop takes 2.7 ms in the cluster and 3.0 ms there in mixed precision,
+// 7.9 and 8.5 ms in float64 (larger ones do not fit); a mixed step of 576^2 took
+// 7.6 and 4.7 ms where one of 512^2 took 3.7 and 4.5.
 constexpr int kS2CtaCells = kSolve2dCells / kS2MaxCTAs;
 // Shared memory of a CTA, and what the kernel's static arrays leave of it (the
 // launch asks the kernel itself; this decides the workspace, without a GPU).
