@@ -298,18 +298,27 @@ struct DiagOut {
 };
 
 // Planes per CTA of a kernel that marches cols column tiles in z: the chunk with
-// the least modelled time, max(1, CTAs / slots) (zc + extra), slots the CTAs
-// resident at once and extra the planes' worth of halo and pipeline start that
-// a chunk pays. Many short chunks (8 CTAs per SM and more) pay it several
-// times over: at 128^3 a sweep from x_in takes 29 us with 14-plane chunks and
-// 48 us with 4-plane ones, the direction kernel 20 and 27 us; at 384^3 chunks
-// of 48 to 96 planes differ by 2 %.
-inline int march_zc(long long cols, int nz, long long slots, int extra, int zmax = 64) {
+// the least modelled time, waves (zc + extra), slots the CTAs resident at once
+// and extra the planes' worth of halo and pipeline start that a chunk pays. A
+// last wave of few CTAs takes at least 0.7 of a full one: it is bound by the
+// latency of a plane. Many short chunks (8 CTAs per SM and more) pay extra
+// several times over: at 128^3 a sweep from x_in takes 29 us with 14-plane chunks
+// and 48 us with 4-plane ones, the direction kernel 20 and 27 us. Chunks of 64
+// planes just above one wave cost as much: at 256^3 the outer residual takes 240
+// us with 64 planes (1.12 waves), 189 with 43 (1.68) and 197 with 32, the sweeps 136,
+// 125 and 122. On 13 grids of 128^3 to 384^3 the chunk is within 3 % of the best of
+// 12 measured ones on average, 11 % at worst; with a last wave counted by its
+// share of the slots, and fewer slots than are resident, 6 and 35 %.
+inline int march_zc(long long cols, int nz, long long slots, int extra, int zmax = 56) {
     int best = 2;
     double cost = 1e300;
     for (int zc = 2; zc <= zmax && zc <= nz; ++zc) {
         const long long b = cols * ((nz + zc - 1) / zc);
-        const double w = b > slots ? double(b) / double(slots) : 1.0;
+        double w = 1.0;
+        if (b > slots) {
+            const double last = double(b % slots) / double(slots);
+            w = double(b / slots) + (last > 0.0 && last < 0.7 ? 0.7 : last);
+        }
         const double c = w * double(zc + extra);
         if (c <= cost) {
             cost = c;

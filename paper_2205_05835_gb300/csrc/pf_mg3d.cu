@@ -835,7 +835,7 @@ void launch_ir_residual3d(const Dims& g, const float* x, const float* b, const f
     a.rb = rb;
     a.sc = sc;
     const long long cols = (long long)((g.nx + 31) / 32) * ((g.ny + 7) / 8);
-    int zc = march_zc(cols, g.nz, 5 * 152, 6);
+    int zc = march_zc(cols, g.nz, 6 * 152, 6);   // (40 registers: six CTAs an SM)
     if (3 * cols * ((g.nz + zc - 1) / zc) > kRedPart) zc = tiled_zc(g);
     a.zc = zc;
     dim3 grid((g.nx + 31) / 32, (g.ny + 7) / 8, (g.nz + zc - 1) / zc);

@@ -242,7 +242,7 @@ void launch_cell_pass_mu3d(const Dims& g, const Phys& ph, const float* phi, floa
 
 int divergence_zc(const Dims& g) {
     const long long cols = (long long)((g.nx + ZX - 1) / ZX) * ((g.ny + ZY - 1) / ZY);
-    return march_zc(cols, g.nz, 6 * 152, 6);
+    return march_zc(cols, g.nz, 8 * 152, 6);   // (32 registers: eight CTAs an SM)
 }
 bool divergence3d_ok(const Dims& g) {
     const int zc = divergence_zc(g);
